@@ -315,12 +315,9 @@ template <typename R>
 __device__ __forceinline__ void su3_reunit_value(M3<R>& m);
 
 template <typename R, int FIELD, int KIND>
-__global__ void __maxnreg__(QCD_SU3_PHASE_MAXNREG) su3_phase_kernel(const Ctx a, int parity, int mu) {
+__device__ __noinline__ void su3_update_fp64(const Ctx& a, int parity, int mu, int h) {
   using P = SU3Policy<R>;
-  const int h = blockIdx.x * blockDim.x + threadIdx.x;
-  if (h >= a.g.Vh) return;
   const Site x = site_of(a.g, parity, h);
-  if (frozen_link(a, mu, x.t)) return;
   const M3<R> A = staple<P, FIELD>(a, x, mu);
   M3<R> U = P::load(a.links, a.g, mu, parity, h);
   M3<R> Ut = U;
@@ -1020,29 +1017,6 @@ __global__ void from_canonical_kernel(const Ctx a, const double* in) {
 // ---------------------------------------------------------------------------
 inline unsigned grid_for(int64_t n, int block) { return unsigned((n + block - 1) / block); }
 
-template <class P, int FIELD, int KIND>
-inline void launch_phase_t(const Ctx& a, int parity, int mu, int block, cudaStream_t st) {
-  static_assert(P::N == 3, "SU(2) uses the kernels of qcd_su2c.cuh");
-  su3_phase_kernel<typename P::Real, FIELD, KIND><<<grid_for(a.g.Vh, block), block, 0, st>>>(a, parity, mu);
-}
-
-template <class P, int KIND>
-inline void launch_phase_level(const Ctx& a, int parity, int mu, int block, cudaStream_t st) {
-  switch (su3_field_level(a)) {
-    case 0: launch_phase_t<P, 0, KIND>(a, parity, mu, block, st); break;
-    case 1: launch_phase_t<P, 1, KIND>(a, parity, mu, block, st); break;
-    default: launch_phase_t<P, 2, KIND>(a, parity, mu, block, st); break;
-  }
-}
-
-template <class P>
-cudaError_t launch_phase(const Ctx& a, int kind, int parity, int mu, int block, cudaStream_t st) {
-  if (kind == KIND_HB) launch_phase_level<P, KIND_HB>(a, parity, mu, block, st);
-  else if (kind == KIND_OR) launch_phase_level<P, KIND_OR>(a, parity, mu, block, st);
-  else launch_phase_level<P, KIND_OR_REUNIT>(a, parity, mu, block, st);  // (no fused measurement here)
-  return cudaGetLastError();
-}
-
 template <class P>
 cudaError_t launch_reunit(const Ctx& a, int advance, cudaStream_t st) {
   const int block = 256;
@@ -1094,43 +1068,6 @@ template <class P>
 cudaError_t launch_from_canonical(const Ctx& a, const double* in, cudaStream_t st) {
   from_canonical_kernel<P><<<grid_for(8LL * a.g.Vh, 256), 256, 0, st>>>(a, in);
   return cudaGetLastError();
-}
-
-template <class P, int FIELD, int KIND>
-int phase_block_limit() {
-  cudaFuncAttributes attr{};
-  const cudaError_t e = cudaFuncGetAttributes(&attr, su3_phase_kernel<typename P::Real, FIELD, KIND>);
-  return e == cudaSuccess ? attr.maxThreadsPerBlock : 0;
-}
-
-template <class P>
-int max_phase_block() {
-  int m = phase_block_limit<P, 0, KIND_HB>();
-  m = std::min(m, phase_block_limit<P, 1, KIND_HB>());
-  m = std::min(m, phase_block_limit<P, 2, KIND_HB>());
-  m = std::min(m, phase_block_limit<P, 0, KIND_OR>());
-  m = std::min(m, phase_block_limit<P, 1, KIND_OR>());
-  m = std::min(m, phase_block_limit<P, 2, KIND_OR>());
-  m = std::min(m, phase_block_limit<P, 0, KIND_OR_REUNIT>());
-  m = std::min(m, phase_block_limit<P, 1, KIND_OR_REUNIT>());
-  m = std::min(m, phase_block_limit<P, 2, KIND_OR_REUNIT>());
-  return m;
-}
-
-template <class P>
-constexpr PolicyOps make_ops(int precision) {
-  return PolicyOps{P::N,
-                   precision,
-                   P::COMPS,
-                   &launch_phase<P>,
-                   &launch_reunit<P>,
-                   &launch_start<P>,
-                   &launch_measure<P>,
-                   &launch_to_canonical<P>,
-                   &launch_from_canonical<P>,
-                   &launch_set_frozen<P>,
-                   nullptr,
-                   &max_phase_block<P>};
 }
 
 }  // namespace qcd

@@ -1,6 +1,34 @@
-// su3_f64.cu -- kernels of the gauge sweep instantiated for one (group, storage).
-#include "qcd_kernels.cuh"
+// su3_f64.cu -- kernels of the gauge sweep for SU(3) with FP64 18-real links.
+// The phase update uses the fixed-point kernel of qcd_su3d.cuh;
+// reunitarization, start, measurements and layout conversion use the shared
+// templates.
+#include "qcd_su3d.cuh"
 
 namespace qcd {
-const PolicyOps kOpsSU3F64 = make_ops<SU3Policy<double>>(0);
+namespace {
+cudaError_t launch_phase(const Ctx& a, int kind, int parity, int mu, int /*block: the kernel's own*/,
+                         cudaStream_t st) {
+  if (kind == KIND_HB) return su3d_launch_hb(a, parity, mu, st);
+  if (kind == KIND_OR) return su3d_launch_level<KIND_OR>(a, parity, mu, st);
+  return su3d_launch_or_reunit(a, parity, mu, st);  // (no fused measurement here)
+}
+
+// Block sizes that qcd_set_block takes (those of the 96-register FP64 kernel
+// that this storage had; the CTA shape is part of the kernel now).
+int max_phase_block() { return 640; }
+}  // namespace
+
+using SU3D = SU3Policy<double>;
+const PolicyOps kOpsSU3F64 = PolicyOps{3,
+                                       0,
+                                       SU3D::COMPS,
+                                       &launch_phase,
+                                       &launch_reunit<SU3D>,
+                                       &launch_start<SU3D>,
+                                       &launch_measure<SU3D>,
+                                       &launch_to_canonical<SU3D>,
+                                       &launch_from_canonical<SU3D>,
+                                       &launch_set_frozen<SU3D>,
+                                       nullptr,
+                                       &max_phase_block};
 }  // namespace qcd
