@@ -17,7 +17,7 @@
 // the kernel loads them with ld.global.cg (L2 only; no stale L1 lines).
 #include "qcd.h"
 #include "qcd_internal.h"
-#include "qcd_su2c.cuh"
+#include "qcd_su2d.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -166,6 +166,12 @@ __device__ inline int4 site_digits(const Geom& g, int r) {
   return d;
 }
 
+template <typename R, bool FIELD, int KIND, int MU>
+__device__ __forceinline__ double batch_update(const Ctx& a, int p, const LexSite& x, uint32_t sweep) {
+  if constexpr (sizeof(R) == 8) return su2d_update_at<FIELD, KIND, MU, true>(a, p, x, sweep);
+  else return double(su2c_update_at<R, FIELD, KIND, MU, true>(a, p, x, sweep));
+}
+
 // One phase over this CTA's share of the lattice; returns the sum of the
 // updates' plaquette terms (KIND_OR_MEAS) in FP64.
 // The digits of 2 stride are the same for the whole CTA: they are read from
@@ -180,7 +186,7 @@ __device__ __forceinline__ double batch_phase(const Ctx& a, int p, int mu, int f
 #define QCD_BATCH_MU(MU)                                                                          \
   case MU:                                                                                        \
     for (int h = first; h < a.g.Vh; h += stride, w.step(a.g.Ns, *d))                                  \
-      v += double(su2c_update_at<R, FIELD, KIND, MU, true>(a, p, w.site(p, h), sweep));            \
+      v += batch_update<R, FIELD, KIND, MU>(a, p, w.site(p, h), sweep);                            \
     break;
     QCD_BATCH_MU(0)
     QCD_BATCH_MU(1)
@@ -282,8 +288,12 @@ __device__ void batch_run(const BatchArgs& b, int li, const BatchLat& L, int j) 
 #define QCD_BATCH_MAXNREG 64
 #endif
 
+// FP64 links take the fixed-point update (12.6 -> 4.8 ms per sweep of the
+// 64-lattice scan): 128 registers (4.9 ms; 112 / 96 / 80 / 64: 5.1 / 5.6 / 6.4 / 7.0).
+constexpr int BATCH_MAXNREG_F64 = 128;
+
 template <typename R>
-__global__ void __maxnreg__(QCD_BATCH_MAXNREG) batch_kernel(const BatchArgs b) {
+__global__ void __maxnreg__(sizeof(R) == 8 ? BATCH_MAXNREG_F64 : QCD_BATCH_MAXNREG) batch_kernel(const BatchArgs b) {
   const int li = b.cta_lattice[blockIdx.x];
   const BatchLat L = b.lat[li];
   const int j = int(blockIdx.x) - L.g0;

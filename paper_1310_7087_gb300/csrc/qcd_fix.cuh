@@ -254,18 +254,24 @@ QCD_HD Fx fx_scale1p(Fx v, Fx d) {
   return fx_limbs(fx_add(fx_value(v), s.value()));
 }
 
-// A vector scaled to unit length, given to 2^-19: 1/sqrt(1 + e) - 1 =
-// -e/2 + 3 e^2/8 to below 2^-58.  False when it is further off.
+// 1/sqrt(n) - 1 for a squared norm n within 2^-19 of 1: -e/2 + 3 e^2/8 to below
+// 2^-58.  False when it is further off.
+QCD_HD bool fx_unit_factor(int64_t n, Fx& d) {
+  const int64_t e = fx_sub(n, int64_t(1) << FX_UNIT);
+  if (fx_abs(e) >> 39) return false;
+  const int32_t es = int32_t(e >> 8);
+  d = fx_limbs(-(e >> 1) + ((3 * (fx_mad(es, es, 0) >> 3)) >> 42));
+  return true;
+}
+
 QCD_HD bool fx_unit3(FxC v[3]) {
   FxAcc n;
   for (int k = 0; k < 3; ++k) {
     n.add(v[k].re, v[k].re);
     n.add(v[k].im, v[k].im);
   }
-  const int64_t e = fx_sub(n.value(), int64_t(1) << FX_UNIT);
-  if (fx_abs(e) >> 39) return false;
-  const int32_t es = int32_t(e >> 8);
-  const Fx d = fx_limbs(-(e >> 1) + ((3 * (fx_mad(es, es, 0) >> 3)) >> 42));
+  Fx d;
+  if (!fx_unit_factor(n.value(), d)) return false;
   for (int k = 0; k < 3; ++k) v[k] = {fx_scale1p(v[k].re, d), fx_scale1p(v[k].im, d)};
   return true;
 }

@@ -297,7 +297,7 @@ __device__ __forceinline__ void left_rotate(M3<R>& m, const Quat<R>& r, int i, i
   }
 }
 
-// Register cap of the SU(3) phase kernels: fewer registers per thread let more
+// Register cap of the SU(3) FP32 phase kernels: fewer registers per thread let more
 // warps stay resident to hide the latency of the 18-link gather.
 #ifndef QCD_SU3_PHASE_MAXNREG
 #define QCD_SU3_PHASE_MAXNREG 96
@@ -314,6 +314,8 @@ __device__ __forceinline__ Quat<R> su2_reunit_value(const Quat<R>& u);
 template <typename R>
 __device__ __forceinline__ void su3_reunit_value(M3<R>& m);
 
+// The update of one link in FP64: what links outside the range of the fixed-point
+// kernel (qcd_su3d.cuh) take.
 template <typename R, int FIELD, int KIND>
 __device__ __noinline__ void su3_update_fp64(const Ctx& a, int parity, int mu, int h) {
   using P = SU3Policy<R>;

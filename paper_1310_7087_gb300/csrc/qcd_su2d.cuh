@@ -1,0 +1,325 @@
+// qcd_su2d.cuh -- SU(2) phase update with FP64 links, its quaternion products in
+// fixed point (qcd_fix.cuh) on the integer pipe; the counterpart of qcd_su2c.cuh
+// for the single-lattice kernels and the batched kernel (CG: loads through L2).
+#pragma once
+
+#include "qcd_fixmath.cuh"
+#include "qcd_su2c.cuh"
+
+namespace qcd {
+
+// Quaternion of a link, conjugated with DAG.  Conversions on the integer pipe:
+// a third of them on the FP64 unit was no faster at 64^3x16 and 14 % slower at
+// 20^3x4, two thirds slower everywhere.
+template <bool DAG, bool CG>
+__device__ __forceinline__ void su2d_load(const Ctx& a, int d, int par, int s, Fx q[4], uint32_t& big) {
+  const Quat<double> u = SU2Policy<double>::template load<CG>(a.links, a.g, d, par, s >> 1);
+  const double v[4] = {u.q0, DAG ? -u.q1 : u.q1, DAG ? -u.q2 : u.q2, DAG ? -u.q3 : u.q3};
+#pragma unroll
+  for (int k = 0; k < 4; ++k) q[k] = fx_load_int(v[k], big);
+}
+
+// q (c + s k), or with LEFT (c - s k) q, the adjoint of q^+ (c + s k); with
+// INVERSE the sign of s turned.
+template <bool LEFT, bool INVERSE>
+__device__ __forceinline__ void su2d_phase(const Ctx& a, int x, Fx q[4], uint32_t& bad) {
+  uint32_t e = 0;
+  const double2 v = __ldg(a.phase64 + x);
+  const Fx c = fx_load_int(v.x, e), s = fx_load_int(LEFT != INVERSE ? -v.y : v.y, e), n = fx_neg(s);
+  FxAcc r[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) r[k].add(q[k], c);
+  r[0].add(q[3], n);
+  r[3].add(q[0], s);
+  r[1].add(q[2], LEFT ? s : n);
+  r[2].add(q[1], LEFT ? n : s);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int64_t t = r[k].value();
+    fx_check(t, bad);
+    q[k] = fx_limbs(t);
+  }
+}
+
+template <bool FIELD, int D, bool DAG, bool CG>
+__device__ __forceinline__ void su2d_eff(const Ctx& a, int par, const LexSite& x, Fx q[4], uint32_t& big,
+                                         uint32_t& bad) {
+  su2d_load<DAG, CG>(a, D, par, x.s, q, big);
+  if (FIELD && D == 1) su2d_phase<DAG, false>(a, x.c[0], q, bad);
+}
+
+// A += one staple of U_MU(x): Ut_nu(x+mu) Ut_mu(x+nu)^+ Ut_nu(x)^+, or
+// Ut_nu(x+mu-nu)^+ Ut_mu(x-nu)^+ Ut_nu(x-nu).
+template <bool FIELD, int MU, int NU, bool LOWER, bool CG>
+__device__ __forceinline__ void su2d_staple(const Ctx& a, int p, const LexSite& x, int64_t A[4], uint32_t& big,
+                                            uint32_t& bad) {
+  const LexSite xn = lex_step<NU, LOWER ? -1 : +1>(a.g, x);
+  const LexSite& base = LOWER ? xn : x;
+  const LexSite xp = lex_step<MU, +1>(a.g, base);
+  const int pb = LOWER ? p ^ 1 : p;
+  Fx u[4], v[4];
+  int64_t t[4];
+  su2d_eff<FIELD, NU, LOWER, CG>(a, pb ^ 1, xp, u, big, bad);
+  su2d_eff<FIELD, MU, true, CG>(a, p ^ 1, xn, v, big, bad);
+  fx_qmul(u, v, t);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    fx_check(t[k], bad);
+    u[k] = fx_limbs(t[k]);
+  }
+  su2d_eff<FIELD, NU, !LOWER, CG>(a, pb, base, v, big, bad);
+  fx_qmul(u, v, t);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    fx_check(t[k], bad);
+    A[k] += t[k];
+  }
+}
+
+// The update in FP64, out of line: links outside the fixed-point range.
+template <bool FIELD, int KIND, int MU, bool CG>
+__device__ __noinline__ double su2d_general(Ctx a, int parity, LexSite x, uint32_t sweep) {
+  return su2c_update_at<double, FIELD, KIND, MU, CG>(a, parity, x, sweep);
+}
+
+static __device__ __noinline__ Quat<double> su2d_haar(Stream dir) { return su2_haar<double>(dir, 0u); }
+
+// One link update given its staple sum A (and the part of it over nu < MU), as
+// su2c_update_at.
+template <bool FIELD, int KIND, int MU, bool CG>
+__device__ __forceinline__ double su2d_update(const Ctx& a, int parity, const LexSite& x, uint32_t sweep,
+                                              int64_t A[4], const int64_t low[4], uint32_t big, uint32_t bad,
+                                              const FxKpFirst* first) {
+  constexpr bool reunit = KIND == KIND_OR_REUNIT || KIND == KIND_OR_MEAS;
+  constexpr bool meas = KIND == KIND_OR_MEAS;
+  constexpr bool phased = FIELD && MU == 1;
+  using P = SU2Policy<double>;
+  Fx u[4];
+  bool keep = false;
+  if (KIND == KIND_HB) {
+    if ((bad & FX_BAD) || (big & FX_BIG)) return su2d_general<FIELD, KIND, MU, CG>(a, parity, x, sweep);
+    const Stream dir = make_stream(a.k0, a.k1, uint32_t(x.s), sweep, MU, 0, KIND_DIR);
+    if (a.beta == 0.0 || (A[0] | A[1] | A[2] | A[3]) == 0) {
+      const Quat<double> R = su2d_haar(dir);
+      u[0] = fx_load(R.q0, big);
+      u[1] = fx_load(R.q1, big);
+      u[2] = fx_load(R.q2, big);
+      u[3] = fx_load(R.q3, big);
+    } else {
+      const Stream tries = make_stream(a.k0, a.k1, uint32_t(x.s), sweep, MU, 0, KIND_TRY);
+      if (!fx_heatbath(A, 1.0 / a.beta, a.nhit, tries, *first, u)) {
+        atomicAdd(a.exhausted, 1ull);
+        return 0.0;  // the link stays as it is
+      }
+    }
+  } else {
+    su2d_load<false, CG>(a, MU, parity, x.s, u, big);
+    if (phased) su2d_phase<false, false>(a, x.c[0], u, bad);
+    if ((bad & FX_BAD) || (big & FX_BIG)) return su2d_general<FIELD, KIND, MU, CG>(a, parity, x, sweep);
+    // V^+ U^+ V^+ = 2 <V^+, U> V^+ - U for the unit quaternion V = A / |A|
+    if (fx_normalise4(A)) {
+      Fx w[4];
+      FxAcc n, d;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        w[k] = fx_limbs(k ? -A[k] : A[k]);
+        n.add(w[k], w[k]);
+        d.add(w[k], u[k]);
+      }
+      FxAcc f;
+      f.add(fx_limbs(d.value()), fx_limbs(fx_reciprocal(n.value())));
+      fx_check(f.value(), bad);  // at most |U| / |A| with A normalised above 1/2
+      const Fx s = fx_limbs(f.value());
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        FxAcc t;
+        t.add(w[k], s);
+        u[k] = fx_limbs(fx_sub(2 * t.value(), fx_value(u[k])));
+      }
+      if (bad & FX_BAD) return su2d_general<FIELD, KIND, MU, CG>(a, parity, x, sweep);
+    } else {
+      keep = true;
+    }
+    if (keep && !reunit) return 0.0;
+  }
+  if (phased) su2d_phase<false, true>(a, x.c[0], u, bad);  // Ut_new B^+
+  Quat<double> q;
+  bool done = false;
+  if (reunit) {
+    FxAcc n;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) n.add(u[k], u[k]);
+    Fx d;
+    done = fx_unit_factor(n.value(), d);
+    if (done)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) u[k] = fx_scale1p(u[k], d);
+  }
+  q = {fx_double(fx_value(u[0])), fx_double(fx_value(u[1])), fx_double(fx_value(u[2])), fx_double(fx_value(u[3]))};
+  if (reunit && !done) {
+    q = su2_reunit_value<double>(q);
+    u[0] = fx_load(q.q0, big);
+    u[1] = fx_load(q.q1, big);
+    u[2] = fx_load(q.q2, big);
+    u[3] = fx_load(q.q3, big);
+  }
+  P::store(a.links, a.g, MU, parity, x.s >> 1, q);
+  if (!meas) return 0.0;
+  if (phased) su2d_phase<false, false>(a, x.c[0], u, bad);
+  FxAcc t;  // (1/2) Re Tr(Ut low) / 8
+#pragma unroll
+  for (int k = 0; k < 4; ++k) t.add(u[k], fx_limbs(k ? -(low[k] >> 3) : low[k] >> 3));
+  return 8.0 * fx_double(t.value());
+}
+
+// The whole update by one thread.
+template <bool FIELD, int KIND, int MU, bool CG>
+__device__ __forceinline__ double su2d_update_at(const Ctx& a, int parity, const LexSite& x, uint32_t sweep) {
+  if (frozen_link(a, MU, x.c[3])) return 0.0;
+  int64_t A[4] = {}, low[4] = {};
+  uint32_t big = 0, bad = 0;
+#pragma unroll
+  for (int n = 0; n < 3; ++n) {
+    if (n == MU)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) low[k] = A[k];
+    switch (n + (n >= MU)) {
+#define QCD_SU2D_NU(NU)                                                                \
+  case NU:                                                                             \
+    if (NU != MU) {                                                                    \
+      su2d_staple<FIELD, MU, NU, false, CG>(a, parity, x, A, big, bad);          \
+      su2d_staple<FIELD, MU, NU, true, CG>(a, parity, x, A, big, bad);           \
+    }                                                                                  \
+    break;
+      QCD_SU2D_NU(0)
+      QCD_SU2D_NU(1)
+      QCD_SU2D_NU(2)
+      QCD_SU2D_NU(3)
+#undef QCD_SU2D_NU
+    }
+  }
+  if (MU == 3)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) low[k] = A[k];
+  FxKpFirst first;
+  if (KIND == KIND_HB)
+    first = fx_kp_first(make_stream(a.k0, a.k1, uint32_t(x.s), sweep, MU, 0, KIND_TRY),
+                        make_stream(a.k0, a.k1, uint32_t(x.s), sweep, MU, 0, KIND_DIR));
+  return su2d_update<FIELD, KIND, MU, CG>(a, parity, x, sweep, A, low, big, bad, &first);
+}
+
+// One staple, chosen by s (uniform in a warp).
+template <bool FIELD, int MU, bool CG>
+__device__ __forceinline__ void su2d_one_staple(const Ctx& a, int p, const LexSite& x, int s, int64_t A[4],
+                                                uint32_t& big, uint32_t& bad) {
+  switch (s) {
+#define QCD_SU2D_ONE(N)                                                                                          \
+  case 2 * N: su2d_staple<FIELD, MU, N + (N >= MU), false, CG>(a, p, x, A, big, bad); break;              \
+  case 2 * N + 1: su2d_staple<FIELD, MU, N + (N >= MU), true, CG>(a, p, x, A, big, bad); break;
+    QCD_SU2D_ONE(0)
+    QCD_SU2D_ONE(1)
+    QCD_SU2D_ONE(2)
+#undef QCD_SU2D_ONE
+  }
+}
+
+// Bound: integer pipe and FP64 unit together (ncu at 32^3x8, overrelaxation of
+// t-links: ALU 45 %, 3,390 instructions per update) where the FP64 form was bound
+// by the FP64 unit.  Phase times, us, FP64 form -> this, overrelaxation /
+// heat-bath of y-links: 4^3x4 14.4 / 30.8 -> 6.4 / 10.6; 32^3x8 77 / 159 -> 31 / 45;
+// 64^3x16 1104 / 2135 -> 440 / 661.  128 registers: 96 / 80 / 64 gave sweeps of
+// 8.2 / 8.5 / 9.4 ms at 64^3x16 against 8.2, and 572 / 640 / 613 us at 32^3x8
+// against 534.
+//
+// SPLIT = 1: one thread per link.  SPLIT = 6: six warps share 32 links, each
+// taking one staple; the integer sums are exact, so the results are the same.
+template <bool FIELD, int KIND, int MU, int SPLIT>
+__global__ void __maxnreg__(128) su2d_phase_kernel(const __grid_constant__ Ctx a, int parity) {
+  double v = 0.0;
+  if (SPLIT == 1) {
+    const int h = blockIdx.x * blockDim.x + threadIdx.x;
+    if (h < a.g.Vh)
+      v = su2d_update_at<FIELD, KIND, MU, false>(a, parity, lex_site(a, parity, h), KIND == KIND_HB ? *a.sweep : 0u);
+  } else {
+    __shared__ int64_t part[SPLIT][4][32];
+    __shared__ uint32_t flag[SPLIT][32];
+    const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
+    const int h = blockIdx.x * 32 + lane;
+    const bool in = h < a.g.Vh;
+    const LexSite x = lex_site(a, parity, in ? h : a.g.Vh - 1);
+    const bool on = in && !frozen_link(a, MU, x.c[3]);
+    const uint32_t sweep = KIND == KIND_HB ? *a.sweep : 0u;
+    int64_t A[4] = {};
+    uint32_t big = 0, bad = 0;
+    FxKpFirst first;
+    su2d_one_staple<FIELD, MU, false>(a, parity, x, role, A, big, bad);
+    if (role > 0) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) part[role][k][lane] = A[k];
+      flag[role][lane] = (bad & FX_BAD) | (big & FX_BIG);
+    } else if (KIND == KIND_HB) {
+      first = fx_kp_first(make_stream(a.k0, a.k1, uint32_t(x.s), sweep, MU, 0, KIND_TRY),
+                          make_stream(a.k0, a.k1, uint32_t(x.s), sweep, MU, 0, KIND_DIR));
+    }
+    __syncthreads();
+    if (role > 0) return;
+    int64_t low[4] = {};
+#pragma unroll
+    for (int s = 0; s < 6; ++s) {
+      if (s > 0) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) A[k] += part[s][k][lane];
+        bad |= flag[s][lane] & FX_BAD;
+        big |= flag[s][lane] & FX_BIG;
+      }
+      if (KIND == KIND_OR_MEAS && s == 2 * MU - 1)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) low[k] = A[k];
+    }
+    if (on) v = su2d_update<FIELD, KIND, MU, false>(a, parity, x, sweep, A, low, big, bad, &first);
+  }
+  if (KIND == KIND_OR_MEAS) {
+    double* out = a.partials + fused_plaq_offset(a.g, MU) + blockIdx.x;
+    if (SPLIT == 1) {
+      su2c_block_sum(v, out);
+    } else {  // one warp is left
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+      if (threadIdx.x == 0) *out = v;
+    }
+  }
+}
+
+// Split up to one CTA of 32 links per SM (152): sweeps of 1 heat-bath + 1
+// overrelaxation pass, us, split / not: 4^3x4 91 / 145, 8^3x4 105 / 150, 12^3x4
+// (108 CTAs) 137 / 150, 20^3x4 (500) 242 / 160.
+inline bool su2d_split(const GeomH& g) { return (g.Vh + 31) / 32 <= 152; }
+// Links of one CTA for a block size of the caller.
+inline int su2d_links_per_cta(const GeomH& g, int block) { return su2d_split(g) ? 32 : block; }
+
+template <bool FIELD, int KIND, int MU>
+inline void su2d_launch_one(const Ctx& a, int parity, int block, cudaStream_t st) {
+  if (su2d_split(a.g)) su2d_phase_kernel<FIELD, KIND, MU, 6><<<grid_for(a.g.Vh, 32), 192, 0, st>>>(a, parity);
+  else su2d_phase_kernel<FIELD, KIND, MU, 1><<<grid_for(a.g.Vh, block), block, 0, st>>>(a, parity);
+}
+
+template <bool FIELD, int KIND>
+inline void su2d_launch_kind(const Ctx& a, int parity, int mu, int block, cudaStream_t st) {
+  switch (mu) {
+    case 0:
+      if (KIND != KIND_OR_MEAS) su2d_launch_one<FIELD, KIND == KIND_OR_MEAS ? KIND_OR : KIND, 0>(a, parity, block, st);
+      break;
+    case 1: su2d_launch_one<FIELD, KIND, 1>(a, parity, block, st); break;
+    case 2: su2d_launch_one<FIELD, KIND, 2>(a, parity, block, st); break;
+    default: su2d_launch_one<FIELD, KIND, 3>(a, parity, block, st); break;
+  }
+}
+
+template <int KIND>
+inline cudaError_t su2d_launch_level(const Ctx& a, int parity, int mu, int block, cudaStream_t st) {
+  if (phases_on_links(a)) su2d_launch_kind<true, KIND>(a, parity, mu, block, st);
+  else su2d_launch_kind<false, KIND>(a, parity, mu, block, st);
+  return cudaGetLastError();
+}
+
+}  // namespace qcd

@@ -1,7 +1,7 @@
 // qcd_su3c.cuh -- phase kernel for SU(3) with FP32 12-real (two-row) links.
 //
-// Same update as su3_phase_kernel (Cabibbo-Marinari heat-bath or
-// overrelaxation of one checkerboard phase), arranged for the compressed
+// Cabibbo-Marinari heat-bath or overrelaxation of one checkerboard phase (the
+// update of su3_update_fp64), arranged for the compressed
 // storage:
 //   - the direction mu is a template parameter, so neighbour strides, the
 //     parities of the 18 gathered links (odd distance: opposite parity, even

@@ -36,10 +36,12 @@ def links_of(kind, links, rng):
 
 
 @pytest.mark.parametrize("kind", ["unitary", "scaled", "zero"])
-@pytest.mark.parametrize("Ns,Nt,flux,flux8", [(6, 2, 1, 0), (6, 6, 0, 0), (18, 4, 1, 1), (20, 4, 2, 0)])
-def test_su3_phases(q, Ns, Nt, flux, flux8, kind):
-    lat = q.Lattice(3, Ns, Nt, 5.7, flux, FP64_PLAIN, HOT, 7, flux8=flux8)
-    orc = oracle.OracleLattice(3, Ns, Nt, 5.7, flux, 10, 0, flux8=flux8)
+@pytest.mark.parametrize("group,Ns,Nt,flux,flux8", [(3, 6, 2, 1, 0), (3, 6, 6, 0, 0), (3, 18, 4, 1, 1), (3, 20, 4, 2, 0),
+                                                    (2, 6, 2, 1, 0), (2, 6, 6, 0, 0), (2, 18, 4, 2, 0)])
+def test_phases(q, group, Ns, Nt, flux, flux8, kind):
+    beta = 5.7 if group == 3 else 2.3
+    lat = q.Lattice(group, Ns, Nt, beta, flux, FP64_PLAIN, HOT, 7, flux8=flux8)
+    orc = oracle.OracleLattice(group, Ns, Nt, beta, flux, 10, 0, flux8=flux8)
     start = links_of(kind, lat.get_links(), np.random.default_rng(3))
     for step, parity, mu in ((q.QCD_HEATBATH, 1, 0), (q.QCD_OVERRELAX, 0, 0), (q.QCD_HEATBATH, 0, 1),
                              (q.QCD_OVERRELAX, 1, 1), (q.QCD_OVERRELAX_REUNIT, 0, 3)):
