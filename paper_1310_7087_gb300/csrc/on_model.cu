@@ -110,8 +110,186 @@ __device__ __forceinline__ void add_neighbours(const OnCtx& a, int par, const Le
   for (int c = 0; c < 4; ++c) F[c] += v[c];
 }
 
+// The hits of one FP32 site visit, on the words of proposal blocks drawn ahead.
+template <int N>
+struct OnHitsF32 {
+  float phi[4], F[4], two_kappa, lambda, delta, cur;
+  __device__ __forceinline__ OnHitsF32(const OnCtx& a, const float p[4], const float f[4])
+      : two_kappa(float(2.0 * a.kappa)), lambda(float(a.lambda)), delta(float(a.delta)) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      phi[c] = p[c];
+      F[c] = f[c];
+    }
+    cur = local_action<float, N>(phi, F, two_kappa, lambda);
+  }
+  __device__ __forceinline__ bool hit(const uint4& w, uint32_t aw) {
+    const uint32_t wu[4] = {w.x, w.y, w.z, w.w};
+    float trial[4] = {phi[0], phi[1], phi[2], phi[3]};
+#pragma unroll
+    for (int c = 0; c < N; ++c) trial[c] = fma(delta, fma(2.f, u01<float>(wu[c]), -1.f), phi[c]);
+    const float next = local_action<float, N>(trial, F, two_kappa, lambda);
+    const float dS = next - cur;
+    if (!(dS <= 0.f || u01<float>(aw) < q_exp(-dS))) return false;
+#pragma unroll
+    for (int c = 0; c < N; ++c) phi[c] = trial[c];
+    cur = next;
+    return true;
+  }
+  __device__ __forceinline__ void flush() {}
+};
+
+// The Metropolis test in FP64 on phi = phi0 + delta K, trial = phi0 + delta T
+// (delta in units of the steps' 2^-23), out of line: the FP32 test below leaves
+// about one hit in a few thousand to it.
+struct OnSite64 {
+  double phi0[4], F[4];
+};
+struct OnSteps {
+  int k[4], t[4];
+};
+template <int N>
+__device__ __noinline__ bool on_test_fp64(OnSite64 s, OnSteps n, double two_kappa, double lambda, double step,
+                                          uint32_t aw) {
+  double phi[4], trial[4];
+#pragma unroll
+  for (int c = 0; c < N; ++c) {
+    phi[c] = fma(step, double(n.k[c]), s.phi0[c]);
+    trial[c] = fma(step, double(n.t[c]), s.phi0[c]);
+  }
+  const double dS = local_action<double, N>(trial, s.F, two_kappa, lambda) -
+                    local_action<double, N>(phi, s.F, two_kappa, lambda);
+  return dS <= 0.0 || u01<double>(aw) < q_exp(-dS);
+}
+
+// The hits of one FP64 site visit without FP64 arithmetic in the loop (an FP64
+// instruction takes a warp 64 cycles; a hit took about 50 of them).  A proposal
+// moves phi by delta (2u - 1) = delta 2^-23 k with an odd integer k, so accepted
+// moves are summed as integers, and the new phi is phi0 + delta 2^-23 K, rounded
+// once (in place of once per accepted hit).  The test u < exp(-dS) is decided
+// in FP32 where its error bound allows:
+//   dS = -2 kappa e.F + q (1 + lambda (2 P + q - 2)),  e = trial - phi,
+//   q = e.(phi + trial), P = phi.phi;
+// with W_c = 2 (|phi_c| + |phi0_c| + delta), which bounds |phi_c| + |trial_c| and,
+// times 1.5 2^-24, the error of either, the roundings of 2^-24 add up to less than
+// 16 2^-24 of
+//   2 kappa a1 + a2 (1 + lambda (2 P + 2 + a2)) + lambda |q| sum W^2,
+//   a1 = sum |e F|, a2 = sum |e| W (absolute values throughout),
+// eps below; exp adds (4 + 2 |dS|) 2^-23.  Otherwise the test is taken in FP64.
+// Infinities and NaN fail both comparisons and go there too.
+template <int N>
+struct OnHitsF64 {
+  OnSite64 site;
+  double two_kappa, lambda, step;
+  float p0[4], p[4], F[4], W[4], kf, lf, sf, df, P, w2;
+  int K[4];
+  __device__ __forceinline__ OnHitsF64(const OnCtx& a, const double phi[4], const double f[4])
+      : two_kappa(2.0 * a.kappa), lambda(a.lambda), step(a.delta * 0x1p-23) {
+    kf = float(two_kappa);
+    lf = float(lambda);
+    sf = float(step);
+    df = fabsf(float(a.delta));
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      site.phi0[c] = phi[c];
+      site.F[c] = f[c];
+      F[c] = float(f[c]);
+    }
+    restart();
+  }
+  __device__ __forceinline__ void restart() {
+#pragma unroll
+    for (int c = 0; c < N; ++c) {
+      K[c] = 0;
+      p0[c] = p[c] = float(site.phi0[c]);
+    }
+    bound();
+  }
+  __device__ __forceinline__ void bound() {
+    w2 = 0.f;
+    P = 0.f;
+#pragma unroll
+    for (int c = 0; c < N; ++c) {
+      W[c] = 2.f * (fabsf(p[c]) + (fabsf(p0[c]) + df));
+      w2 = fmaf(W[c], W[c], w2);
+      P = fmaf(p[c], p[c], P);
+    }
+  }
+  __device__ __forceinline__ bool hit(const uint4& w, uint32_t aw) {
+    const uint32_t wu[4] = {w.x, w.y, w.z, w.w};
+    float t[4], s1 = 0.f, q = 0.f, a1 = 0.f, a2 = 0.f;
+    int T[4];
+#pragma unroll
+    for (int c = 0; c < N; ++c) {
+      const int k = int((wu[c] >> 8) | 1u) - (1 << 23);
+      T[c] = K[c] + k;
+      t[c] = fmaf(sf, float(T[c]), p0[c]);
+      const float e = sf * float(k);
+      s1 = fmaf(e, F[c], s1);
+      q = fmaf(e, p[c] + t[c], q);
+      a1 = fmaf(fabsf(e), fabsf(F[c]), a1);
+      a2 = fmaf(fabsf(e), W[c], a2);
+    }
+    const float x = fmaf(kf, s1, -q * fmaf(lf, fmaf(2.f, P, q) - 2.f, 1.f));
+    const float E = __expf(x), u = u01<float>(aw);
+    const float l = fabsf(lf);
+    const float eps = 0x1p-20f * (fabsf(kf) * a1 + fmaf(a2, fmaf(l, fmaf(2.f, P, a2) + 2.f, 1.f), l * fabsf(q) * w2));
+    const float m = fmaf(fabsf(x), 0x1p-22f, fmaf(2.f, eps, 0x1p-21f));
+    bool yes = u < fmaf(-E, m, E);
+    if (!yes && !(eps < 1.f && u > fmaf(E, m, E))) {
+      OnSteps n;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        n.k[c] = c < N ? K[c] : 0;
+        n.t[c] = c < N ? T[c] : 0;
+      }
+      yes = on_test_fp64<N>(site, n, two_kappa, lambda, step, aw);
+    }
+    if (!yes) return false;
+#pragma unroll
+    for (int c = 0; c < N; ++c) {
+      K[c] = T[c];
+      p[c] = t[c];
+    }
+    bound();
+    return true;
+  }
+  // Every 128 hits at most: |K| stays below 2^30.
+  __device__ __forceinline__ void flush() {
+#pragma unroll
+    for (int c = 0; c < N; ++c) site.phi0[c] = fma(step, double(K[c]), site.phi0[c]);
+    restart();
+  }
+};
+
 template <typename R, int N>
-__global__ void on_phase_kernel(const OnCtx a, int parity) {
+struct OnHits;
+template <int N>
+struct OnHits<float, N> : OnHitsF32<N> {
+  using OnHitsF32<N>::OnHitsF32;
+  __device__ __forceinline__ void result(float v[4]) const {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v[c] = this->phi[c];
+  }
+};
+template <int N>
+struct OnHits<double, N> : OnHitsF64<N> {
+  using OnHitsF64<N>::OnHitsF64;
+  __device__ __forceinline__ void result(double v[4]) const {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v[c] = this->site.phi0[c];
+  }
+};
+
+// Blocks of up to 512 threads have to launch: 128 registers at most.  A sweep of
+// O(4) with 100 hits per site, us, before -> now: FP32 8^3x8 55.9 -> 49.8, 32^4
+// 456 -> 447 (80 registers; 64: 473, 128: 452); FP64 8^3x8 363 -> 85, 16^4 655 ->
+// 105, 32^4 8649 -> 873.  Bound: the integer pipe (1.25 Philox blocks per hit, 160
+// cycles of an SM sub-partition per warp and hit in FP32), at small sizes the
+// latency of one hit after another.
+constexpr int ON_MAXNREG_F32 = 80, ON_MAXNREG_F64 = 128;
+template <typename R, int N>
+__global__ void __maxnreg__(sizeof(R) == 4 ? ON_MAXNREG_F32 : ON_MAXNREG_F64) on_phase_kernel(const OnCtx a, int parity) {
   const int h = blockIdx.x * blockDim.x + threadIdx.x;
   unsigned n_acc = 0;
   if (h < a.g.Vh) {
@@ -129,28 +307,30 @@ __global__ void on_phase_kernel(const OnCtx a, int parity) {
     add_neighbours<R, 3>(a, parity ^ 1, x, F);
     R phi[4];
     OnStore<R>::load(a, parity, h, phi);
-    const R two_kappa = R(2.0 * a.kappa), lambda = R(a.lambda), delta = R(a.delta);
-    R cur = local_action<R, N>(phi, F, two_kappa, lambda);
+    OnHits<R, N> site(a, phi, F);
     const uint32_t sweep = *a.sweep;
-    uint4 acc = make_uint4(0u, 0u, 0u, 0u);
-    for (int hit = 0; hit < a.nhit; ++hit) {
-      const uint4 w = philox4x32_10(make_uint4(uint32_t(x.s), sweep, KIND_ON_PROPOSE << 4, uint32_t(hit)), a.k0, a.k1);
-      if ((hit & 3) == 0)
-        acc = philox4x32_10(make_uint4(uint32_t(x.s), sweep, KIND_ON_ACCEPT << 4, uint32_t(hit >> 2)), a.k0, a.k1);
-      const uint32_t wu[4] = {w.x, w.y, w.z, w.w};
-      R trial[4] = {phi[0], phi[1], phi[2], phi[3]};
+    // Four hits share an acceptance block; their four proposal blocks are drawn
+    // with it, five independent Philox chains in flight.
+    for (int hit = 0; hit < a.nhit; hit += 4) {
+      const uint4 acc =
+          philox4x32_10(make_uint4(uint32_t(x.s), sweep, KIND_ON_ACCEPT << 4, uint32_t(hit >> 2)), a.k0, a.k1);
+      uint4 w[4];
 #pragma unroll
-      for (int c = 0; c < N; ++c) trial[c] = fma(delta, fma(R(2), u01<R>(wu[c]), R(-1)), phi[c]);
-      const R next = local_action<R, N>(trial, F, two_kappa, lambda);
-      const R dS = next - cur;
-      const uint32_t aw = (hit & 3) == 0 ? acc.x : (hit & 3) == 1 ? acc.y : (hit & 3) == 2 ? acc.z : acc.w;
-      if (dS <= R(0) || u01<R>(aw) < q_exp(-dS)) {
+      for (int j = 0; j < 4; ++j)
+        w[j] = philox4x32_10(make_uint4(uint32_t(x.s), sweep, KIND_ON_PROPOSE << 4, uint32_t(hit + j)), a.k0, a.k1);
+      const uint32_t aw[4] = {acc.x, acc.y, acc.z, acc.w};
+      if (hit + 4 <= a.nhit) {
 #pragma unroll
-        for (int c = 0; c < N; ++c) phi[c] = trial[c];
-        cur = next;
-        ++n_acc;
+        for (int j = 0; j < 4; ++j) n_acc += site.hit(w[j], aw[j]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+          if (hit + j < a.nhit) n_acc += site.hit(w[j], aw[j]);
       }
+      if ((hit & 127) == 124) site.flush();
     }
+    site.flush();
+    site.result(phi);
     OnStore<R>::store(a, parity, h, phi);
   }
   // one atomic per warp for the acceptance count
