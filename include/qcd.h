@@ -174,12 +174,12 @@ int qcd_sweep(qcd_lattice *lat, int n_heatbath, int n_overrelax, uint64_t seed);
 /* A working sweep (sec. 4: a sweep followed by measurements): n_heatbath
  * sweeps as qcd_sweep, then the plaquette and Polyakov loop of the resulting
  * configuration into host_out[5] = {P, P_s, P_t, Re L, Im L} (as
- * qcd_measure).  With n_overrelax >= 1, FP32 SU(3) storage and the
- * effective-link field mode, the plaquette sums are fused into the last
+ * qcd_measure).  With n_overrelax >= 1 and the effective-link field mode,
+ * the plaquette sums are fused into the last
  * overrelaxation pass: after the pass each plaquette of plane (mu, nu < mu)
  * contains exactly one odd mu-link, so the odd phases mu = 1, 2, 3 add
  * Re Tr(Ut A_nu) for nu < mu over their updated links (A_nu the staples of
- * plane (mu, nu); each warp adds its threads' FP32 values by error-free
+ * plane (mu, nu); FP32: each warp adds its threads' values by error-free
  * TwoSum and finishes in FP64, the block adds its warps in FP64, and the final
  * sums take the 1/3) and no separate pass over the links is needed; otherwise
  * the measurement kernels run after the sweeps.  wait = 1: returns after the
@@ -205,8 +205,8 @@ int qcd_working_sweep(qcd_lattice *lat, int n_heatbath, int n_overrelax,
  *                                 lattice's measurement scratch (the SU(3)
  *                                 1/3 is taken in the final sums);
  *                                 QCD_ERR_NOT_SUPPORTED
- *                                 where qcd_working_sweep does not fuse its
- *                                 measurement (FP64 SU(3), frozen mode).
+ *                                 for FP64 SU(3) storage and in the frozen
+ *                                 mode.
  * After the eight phases of a last pass run this way (QCD_OVERRELAX_REUNIT for
  * parity 0 and for (1, 0), QCD_OVERRELAX_MEASURE for (1, 1..3)),
  * qcd_measure_fused_finish returns the working sweep's measurement. */

@@ -643,6 +643,11 @@ static bool fused_measure_available(const qcd_lattice* L) {
   return L->ops->measure_fused_tail != nullptr && L->field_mode == QCD_FIELD_LINKS;
 }
 
+// Where the fused measurement can also be driven phase by phase.
+static bool fused_measure_by_phase(const qcd_lattice* L) {
+  return fused_measure_available(L) && !(L->group == 3 && L->precision == QCD_FP64_PLAIN);
+}
+
 static int measure_impl(qcd_lattice* L, int effective, double* plaq, double* poly);
 
 int qcd_working_sweep(qcd_lattice* L, int n_heatbath, int n_overrelax, uint64_t seed, double* host_out, int wait) {
@@ -679,7 +684,7 @@ int qcd_phase(qcd_lattice* L, int kind, int parity, int mu, uint64_t seed) {
       return set_error(QCD_ERR_INVALID_ARG,
                        "QCD_OVERRELAX_MEASURE is a phase of odd parity with mu >= 1 (got parity %d, mu %d)",
                        parity, mu);
-    if (!fused_measure_available(L))
+    if (!fused_measure_by_phase(L))
       return set_error(QCD_ERR_NOT_SUPPORTED,
                        "the fused measurement needs FP32 SU(3) or SU(2) storage and the effective-link field mode");
   }
@@ -692,7 +697,7 @@ int qcd_phase(qcd_lattice* L, int kind, int parity, int mu, uint64_t seed) {
 int qcd_measure_fused_finish(qcd_lattice* L, double* host_out) {
   if (int rc = check(L)) return rc;
   if (!host_out) return set_error(QCD_ERR_INVALID_ARG, "host_out is null");
-  if (!fused_measure_available(L))
+  if (!fused_measure_by_phase(L))
     return set_error(QCD_ERR_NOT_SUPPORTED,
                      "the fused measurement needs FP32 SU(3) or SU(2) storage and the effective-link field mode");
   if (int rc = use_device(L)) return rc;

@@ -94,7 +94,12 @@ __host__ __device__ inline int fused_stride(const GeomH& g) { return (g.Vh + 31)
 __host__ __device__ inline int fused_plaq_offset(const GeomH& g, int mu) {
   return 2 * meas_poly_blocks(g) + (mu - 1) * fused_stride(g);
 }
-inline size_t fused_partials(const GeomH& g) { return size_t(fused_plaq_offset(g, 4)); }
+// A tail whose Polyakov-loop blocks take 32 sites (SU(3) FP64) keeps their partials
+// after these.
+__host__ __device__ inline int fused_poly32_blocks(const GeomH& g) {
+  return int(((long long)g.Ns * g.Ns * g.Ns + 31) / 32);
+}
+inline size_t fused_partials(const GeomH& g) { return size_t(fused_plaq_offset(g, 4)) + 2 * size_t(fused_poly32_blocks(g)); }
 
 // Phase kinds: heat-bath, overrelaxation, and overrelaxation whose kernel also
 // reunitarizes each link it updates before storing it (the last pass of a

@@ -246,8 +246,10 @@ __device__ __forceinline__ typename P::Link load_eff(const Ctx& a, int mu, const
 // Staple sum of U_mu(x) on effective links:
 //   A = sum_{nu != mu} Ut_nu(x+mu) Ut_mu(x+nu)^+ Ut_nu(x)^+
 //                    + (Ut_mu(x-nu) Ut_nu(x+mu-nu))^+ Ut_nu(x-nu)
+// *low receives the part of the sum over nu < mu.
 template <class P, int FIELD, bool CG = false>
-__device__ __forceinline__ typename P::Link staple(const Ctx& a, const Site& x, int mu) {
+__device__ __forceinline__ typename P::Link staple(const Ctx& a, const Site& x, int mu,
+                                                   typename P::Link* low = nullptr) {
   using R = typename P::Real;
   using A = Alg<R>;
   typename P::Link acc;
@@ -255,7 +257,10 @@ __device__ __forceinline__ typename P::Link staple(const Ctx& a, const Site& x, 
   const Site xp = step(a.g, x, mu, +1);
 #pragma unroll
   for (int nu = 0; nu < 4; ++nu) {
-    if (nu == mu) continue;
+    if (nu == mu) {
+      if (low) *low = acc;
+      continue;
+    }
     const Site xpn = step(a.g, x, nu, +1);
     const Site xmn = step(a.g, x, nu, -1);
     const Site xpmn = step(a.g, xp, nu, -1);
@@ -315,23 +320,23 @@ template <typename R>
 __device__ __forceinline__ void su3_reunit_value(M3<R>& m);
 
 // The update of one link in FP64: what links outside the range of the fixed-point
-// kernel (qcd_su3d.cuh) take.
+// kernel (qcd_su3d.cuh) take.  KIND_OR_MEAS returns Re Tr of the final effective
+// link with the staples of the planes (mu, nu < mu).
 template <typename R, int FIELD, int KIND>
-__device__ __noinline__ void su3_update_fp64(const Ctx& a, int parity, int mu, int h) {
+__device__ __noinline__ double su3_update_fp64(const Ctx& a, int parity, int mu, int h) {
   using P = SU3Policy<R>;
   const Site x = site_of(a.g, parity, h);
-  const M3<R> A = staple<P, FIELD>(a, x, mu);
+  M3<R> low;
+  const M3<R> A = staple<P, FIELD>(a, x, mu, KIND == KIND_OR_MEAS ? &low : nullptr);
   M3<R> U = P::load(a.links, a.g, mu, parity, h);
-  M3<R> Ut = U;
+  Cx<R> b[3] = {{R(1), R(0)}, {R(1), R(0)}, {R(1), R(0)}};  // the background of this link
   if (FIELD == 1 && mu == 1) {
-    R bc, bs;
-    load_phase<R>(a, x.x, bc, bs);
-    Ut = Alg<R>::right_phase(U, bc, bs);
+    load_phase<R>(a, x.x, b[0].re, b[0].im);
+    b[1] = conj(b[0]);
   } else if (FIELD == 2 && mu == 1) {
-    Cx<R> b[3];
     load_bdiag<R>(a, x.x, b);
-    Ut = right_bdiag(U, b);
   }
+  const M3<R> Ut = FIELD && mu == 1 ? right_bdiag(U, b) : U;
   M3<R> W = m3_mul(Ut, A);
   const uint32_t s = uint32_t(lex(a.g, x));
   uint32_t sweep = 0;
@@ -368,8 +373,10 @@ __device__ __noinline__ void su3_update_fp64(const Ctx& a, int parity, int mu, i
     left_rotate(W, r, i, j);
   }
   if (exhausted) atomicAdd(a.exhausted, (unsigned long long)exhausted);
-  if (KIND == KIND_OR_REUNIT) su3_reunit_value<R>(U);
+  if (KIND == KIND_OR_REUNIT || KIND == KIND_OR_MEAS) su3_reunit_value<R>(U);
   P::store(a.links, a.g, mu, parity, h, U);
+  if (KIND != KIND_OR_MEAS) return 0.0;
+  return double(m3_retrace_mul(FIELD && mu == 1 ? right_bdiag(U, b) : U, low));  // Re Tr(Ut low)
 }
 
 // ---------------------------------------------------------------------------
@@ -885,11 +892,13 @@ static __global__ void __launch_bounds__(FINAL_THREADS)
 // per-thread sums are reduced by warp shuffles and then across the 32 warps,
 // all in a fixed order.
 // plane_scale multiplies the plane sums: 1 when the phase kernels summed
-// (1/N) Re Tr, 1/N when they summed Re Tr.
-static __global__ void __launch_bounds__(FINAL_THREADS) fused_final_kernel(const Ctx a, int grid, double plane_scale) {
+// (1/N) Re Tr, 1/N when they summed Re Tr.  The Polyakov loop's nl block partials
+// lie at poly_offset.
+static __global__ void __launch_bounds__(FINAL_THREADS)
+    fused_final_kernel(const Ctx a, int grid, double plane_scale, int nl, int poly_offset) {
   constexpr int NW = FINAL_THREADS / 32;
   __shared__ double sh[5][NW];
-  const int nl = meas_poly_blocks(a.g);
+  const double* pl = a.partials + poly_offset;
   const double* p1 = a.partials + fused_plaq_offset(a.g, 1);
   const double* p2 = a.partials + fused_plaq_offset(a.g, 2);
   const double* p3 = a.partials + fused_plaq_offset(a.g, 3);
@@ -911,8 +920,8 @@ static __global__ void __launch_bounds__(FINAL_THREADS) fused_final_kernel(const
     s[2] += p3[b];
   }
   for (int c = threadIdx.x; c < nl; c += FINAL_THREADS) {
-    s[3] += a.partials[2 * c];
-    s[4] += a.partials[2 * c + 1];
+    s[3] += pl[2 * c];
+    s[4] += pl[2 * c + 1];
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll

@@ -186,7 +186,7 @@ template <typename R>
 cudaError_t su2c_measure_fused_tail(const Ctx& a, int block, cudaStream_t st) {
   const int nl = meas_poly_blocks(a.g);
   measure_kernel<SU2Policy<R>, 0><<<nl, MEAS_THREADS, 0, st>>>(a, 0);  // Polyakov loop only
-  fused_final_kernel<<<1, FINAL_THREADS, 0, st>>>(a, int(grid_for(a.g.Vh, block)), 1.0);
+  fused_final_kernel<<<1, FINAL_THREADS, 0, st>>>(a, int(grid_for(a.g.Vh, block)), 1.0, nl, 0);
   return cudaGetLastError();
 }
 

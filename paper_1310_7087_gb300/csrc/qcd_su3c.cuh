@@ -520,7 +520,7 @@ static __global__ void __launch_bounds__(MEAS_THREADS) su3c_poly_kernel(const Ct
 
 inline cudaError_t su3c_measure_fused_tail(const Ctx& a, int block, cudaStream_t st) {
   su3c_poly_kernel<<<meas_poly_blocks(a.g), MEAS_THREADS, 0, st>>>(a);
-  fused_final_kernel<<<1, FINAL_THREADS, 0, st>>>(a, int(grid_for(a.g.Vh, block)), 1.0 / 3.0);
+  fused_final_kernel<<<1, FINAL_THREADS, 0, st>>>(a, int(grid_for(a.g.Vh, block)), 1.0 / 3.0, meas_poly_blocks(a.g), 0);
   return cudaGetLastError();
 }
 

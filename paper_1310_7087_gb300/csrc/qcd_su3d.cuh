@@ -20,6 +20,8 @@
 // for both kinds of staple 1665 (instruction cache).
 #pragma once
 
+#include <type_traits>
+
 #include "qcd_fixmath.cuh"
 #include "qcd_kernels.cuh"
 
@@ -107,6 +109,12 @@ struct Su3dShared {
   int offset[4][2][32];                   // of the neighbour's index, forward and backward
   int64_t first[3][5][32];                // a heat-bath's draws ahead of the staples, by subgroup
 };
+// The plane-summing phases keep the part of the staple sum over nu < mu.
+template <int SPLIT>
+struct Su3dMeasShared : Su3dShared<SPLIT> {
+  FxTile low[SPLIT][3][3];
+  double sum[3];
+};
 
 // The rotation of subgroup `sub` from its block in sh.w into sh.r; returns
 // whether all tries of a heat-bath failed.  Out of line: one copy for the three
@@ -156,7 +164,9 @@ template <int FIELD, int KIND, int SPLIT, int INT>
 __global__ void __launch_bounds__(96 * SPLIT, SU3D_CTAS / SPLIT)
     su3d_phase_kernel(const __grid_constant__ Ctx a, int parity, int mu) {
   extern __shared__ __align__(16) unsigned char smem[];
-  Su3dShared<SPLIT>& sh = *reinterpret_cast<Su3dShared<SPLIT>*>(smem);
+  constexpr bool meas = KIND == KIND_OR_MEAS, reunit = KIND == KIND_OR_REUNIT || meas;
+  using Shared = std::conditional_t<meas, Su3dMeasShared<SPLIT>, Su3dShared<SPLIT>>;
+  Shared& sh = *reinterpret_cast<Shared*>(smem);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, group = SPLIT == 1 ? 0 : warp / 3;
   const int role = warp - 3 * group;
   const int h0 = blockIdx.x * 32 + lane, h = min(h0, a.g.Vh - 1);
@@ -249,7 +259,18 @@ __global__ void __launch_bounds__(96 * SPLIT, SU3D_CTAS / SPLIT)
       A[j][0] += re;
       A[j][1] += im;
     }
+    if constexpr (meas)
+      if (nu < mu) {  // the last one leaves the sum so far
+#pragma unroll
+        for (int j = 0; j < 3; ++j) sh.low[group][role][j].put64(lane, A[j]);
+      }
   }
+  if constexpr (meas)
+    if (group >= 2 * mu) {  // no staple with nu < mu here
+      const int64_t zero[2] = {0, 0};
+#pragma unroll
+      for (int j = 0; j < 3; ++j) sh.low[group][role][j].put64(lane, zero);
+    }
   if (SPLIT > 1) {
     bar_96(1 + group);
     if (group > 0) {
@@ -336,53 +357,169 @@ __global__ void __launch_bounds__(96 * SPLIT, SU3D_CTAS / SPLIT)
   }
 
   sh.flag[role][lane] = (bad & FX_BAD) | (big & FX_BIG);
-  if (KIND == KIND_OR_REUNIT) {
+  if (reunit) {
 #pragma unroll
     for (int i = 0; i < 3; ++i) sh.y[0][i][role].put(lane, U[i]);
   }
   bar_96(1);
-  if (!on) return;
-  if (sh.flag[0][lane] | sh.flag[1][lane] | sh.flag[2][lane]) {  // out of the fixed-point range
-    if (role == 0) su3_update_fp64<double, FIELD, KIND>(a, parity, mu, h);
-    return;
+  const bool out_of_range = sh.flag[0][lane] | sh.flag[1][lane] | sh.flag[2][lane];
+  if (!meas && !on) return;
+  double v64 = 0.0;  // Re Tr of an FP64 update
+  if (on && out_of_range) {
+    if (role == 0) v64 = su3_update_fp64<double, FIELD, KIND>(a, parity, mu, h);
+  } else if (on) {
+    if (exhausted) atomicAdd(a.exhausted, (unsigned long long)exhausted);
+    if (!reunit) {
+      double2* out = reinterpret_cast<double2*>(a.links);
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+        out[vidx(a.g, 3 * i + role, mu, parity, h)] =
+            make_double2(fx_double(fx_value(U[i].re)), fx_double(fx_value(U[i].im)));
+    } else if (role == 0) {
+      FxC m[3][3];
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) m[i][k] = sh.y[0][i][k].get(lane);
+      M3<double> d;
+      auto to_double = [&]() {
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+          for (int k = 0; k < 3; ++k) d.e[i][k] = {fx_double(fx_value(m[i][k].re)), fx_double(fx_value(m[i][k].im))};
+      };
+      if (fx_reunit(m)) {
+        to_double();
+      } else {  // rows far from unitary
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+          for (int k = 0; k < 3; ++k) m[i][k] = sh.y[0][i][k].get(lane);
+        to_double();
+        su3d_reunit(d);
+        if (meas)
+#pragma unroll
+          for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) m[i][k] = {fx_load(d.e[i][k].re, big), fx_load(d.e[i][k].im, big)};
+      }
+      SU3Policy<double>::store(a.links, a.g, mu, parity, h, d);
+      if (meas)
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+          for (int k = 0; k < 3; ++k) sh.z[0][i][k].put(lane, m[i][k]);
+    }
   }
-  if (exhausted) atomicAdd(a.exhausted, (unsigned long long)exhausted);
-  double2* out = reinterpret_cast<double2*>(a.links);
-  if (KIND != KIND_OR_REUNIT) {
+  if constexpr (meas) {
+    bar_96(1);
+    // column `role` of the final effective link times row `role` of the partial sum
+    FxAcc p, q;
+    if (on && !out_of_range) {
+      FxC u[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
-      out[vidx(a.g, 3 * i + role, mu, parity, h)] = make_double2(fx_double(fx_value(U[i].re)), fx_double(fx_value(U[i].im)));
-    return;
+      for (int i = 0; i < 3; ++i) u[i] = sh.z[0][i][role].get(lane);
+      if (FIELD && mu == 1 && (FIELD == 2 || role < 2)) {
+        const FxC b = su3d_b<FIELD>(a, x.x, role);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) u[i] = fx_mul<false>(u[i], b, bad);
+      }
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        int64_t t[2] = {0, 0};
+        for (int g = 0; g < SPLIT; ++g) sh.low[g][role][i].add64(lane, t);
+        p.add(u[i].re, fx_limbs(t[0] >> 3));
+        q.add(u[i].im, fx_limbs(t[1] >> 3));
+      }
+    }
+    double s = 8.0 * fx_warp_sum(fx_diff(p, q));
+    if (role == 0 && __any_sync(0xffffffffu, on && out_of_range)) {
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) v64 += __shfl_down_sync(0xffffffffu, v64, off);
+      s += v64;
+    }
+    if (lane == 0) sh.sum[role] = s;
+    bar_96(1);
+    if (threadIdx.x == 0) a.partials[fused_plaq_offset(a.g, mu) + blockIdx.x] = sh.sum[0] + sh.sum[1] + sh.sum[2];
   }
-  if (role > 0) return;
-  FxC m[3][3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) m[i][k] = sh.y[0][i][k].get(lane);
-  M3<double> d;
-  auto to_double = [&]() {
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int k = 0; k < 3; ++k) d.e[i][k] = {fx_double(fx_value(m[i][k].re)), fx_double(fx_value(m[i][k].im))};
+}
+
+// Polyakov loop of a working sweep's fused measurement: three warps per 32 spatial
+// sites, warp r with row r of the running product over t; each converts row r of
+// the next link for the three.  FP64 block partials of (1/3) Tr, in a fixed order.
+// (The plane sums, this kernel and the final sums add 41 us to a sweep of 16^3x4 and
+// 77 to one of 32^3x8; the separate FP64 measurement took 128 and 780.)
+static __global__ void __launch_bounds__(96) su3d_poly_kernel(const __grid_constant__ Ctx a) {
+  __shared__ FxTile tile[2][3][3];
+  __shared__ uint32_t flag[3][32];
+  __shared__ double sum[3][2];
+  const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
+  const int Ns = a.g.Ns, V3 = Ns * Ns * Ns;
+  const int site = blockIdx.x * 32 + lane, s0 = min(site, V3 - 1);
+  const int xyz = s0 % Ns + s0 / Ns % Ns + s0 / (Ns * Ns);
+  const double2* links = reinterpret_cast<const double2*>(a.links) + 6 * a.g.plane;
+  auto row = [&](int t) {
+    const int64_t s = s0 + int64_t(t) * V3;
+    return su3d_row(a, links + ((xyz + t) & 1) * a.g.plane + (s >> 1), role, false);
   };
-  if (fx_reunit(m)) {
-    to_double();
-  } else {  // rows far from unitary
+  uint32_t big = 0, bad = 0;
+  FxC v[3], w[3];
+  su3d_convert<1>(row(0), false, v, big);
+  RawRow next = row(1);
+#pragma unroll 1
+  for (int t = 1; t < a.g.Nt; ++t) {
+    su3d_convert<1>(next, false, w, big);
+    if (t + 1 < a.g.Nt) next = row(t + 1);
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+    for (int k = 0; k < 3; ++k) tile[t & 1][role][k].put(lane, w[k]);
+    __syncthreads();  // (the other buffer's readers passed this one's predecessor)
 #pragma unroll
-      for (int k = 0; k < 3; ++k) m[i][k] = sh.y[0][i][k].get(lane);
-    to_double();
-    su3d_reunit(d);
+    for (int j = 0; j < 3; ++j) {
+      FxDot<false> d;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) d.add(v[k], tile[t & 1][k][j].get(lane));
+      w[j] = d.limbs(bad);
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) v[k] = w[k];
   }
-  SU3Policy<double>::store(a.links, a.g, mu, parity, h, d);
+  flag[role][lane] = (bad & FX_BAD) | (big & FX_BIG);
+  __syncthreads();
+  const bool in = site < V3, out_of_range = flag[0][lane] | flag[1][lane] | flag[2][lane];
+  const FxC d = role == 0 ? v[0] : role == 1 ? v[1] : v[2];
+  const bool fixed = in && !out_of_range;
+  double re = fx_warp_sum(fixed ? fx_value(d.re) : 0), im = fx_warp_sum(fixed ? fx_value(d.im) : 0);
+  if (role == 0 && __any_sync(0xffffffffu, in && out_of_range)) {
+    double v0 = 0.0, v1 = 0.0;
+    if (in && out_of_range) polyakov_site<SU3Policy<double>>(a, site, v0, v1);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      v0 += __shfl_down_sync(0xffffffffu, v0, off);
+      v1 += __shfl_down_sync(0xffffffffu, v1, off);
+    }
+    re += 3.0 * v0;
+    im += 3.0 * v1;
+  }
+  if (lane == 0) {
+    sum[role][0] = re;
+    sum[role][1] = im;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2)
+    a.partials[fused_plaq_offset(a.g, 4) + 2 * blockIdx.x + threadIdx.x] =
+        (sum[0][threadIdx.x] + sum[1][threadIdx.x] + sum[2][threadIdx.x]) / 3.0;
+}
+
+inline cudaError_t su3d_measure_fused_tail(const Ctx& a, int /*block*/, cudaStream_t st) {
+  const int nl = fused_poly32_blocks(a.g);
+  su3d_poly_kernel<<<nl, 96, 0, st>>>(a);
+  fused_final_kernel<<<1, FINAL_THREADS, 0, st>>>(a, (a.g.Vh + 31) / 32, 1.0 / 3.0, nl, fused_plaq_offset(a.g, 4));
+  return cudaGetLastError();
 }
 
 template <int FIELD, int KIND, int SPLIT, int INT>
 inline cudaError_t su3d_launch_one(const Ctx& a, int parity, int mu, cudaStream_t st) {
-  constexpr int bytes = int(sizeof(Su3dShared<SPLIT>));
+  constexpr int bytes = int(KIND == KIND_OR_MEAS ? sizeof(Su3dMeasShared<SPLIT>) : sizeof(Su3dShared<SPLIT>));
   if (bytes > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(su3d_phase_kernel<FIELD, KIND, SPLIT, INT>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -426,5 +563,6 @@ inline cudaError_t su3d_launch_level(const Ctx& a, int parity, int mu, cudaStrea
 // units of their own.
 cudaError_t su3d_launch_hb(const Ctx& a, int parity, int mu, cudaStream_t st);
 cudaError_t su3d_launch_or_reunit(const Ctx& a, int parity, int mu, cudaStream_t st);
+cudaError_t su3d_launch_or_meas(const Ctx& a, int parity, int mu, cudaStream_t st);
 
 }  // namespace qcd

@@ -10,7 +10,8 @@ cudaError_t launch_phase(const Ctx& a, int kind, int parity, int mu, int /*block
                          cudaStream_t st) {
   if (kind == KIND_HB) return su3d_launch_hb(a, parity, mu, st);
   if (kind == KIND_OR) return su3d_launch_level<KIND_OR>(a, parity, mu, st);
-  return su3d_launch_or_reunit(a, parity, mu, st);  // (no fused measurement here)
+  if (kind == KIND_OR_MEAS && mu >= 1) return su3d_launch_or_meas(a, parity, mu, st);
+  return su3d_launch_or_reunit(a, parity, mu, st);
 }
 
 // Block sizes that qcd_set_block takes (those of the 96-register FP64 kernel
@@ -29,6 +30,6 @@ const PolicyOps kOpsSU3F64 = PolicyOps{3,
                                        &launch_to_canonical<SU3D>,
                                        &launch_from_canonical<SU3D>,
                                        &launch_set_frozen<SU3D>,
-                                       nullptr,
+                                       &su3d_measure_fused_tail,
                                        &max_phase_block};
 }  // namespace qcd

@@ -63,3 +63,23 @@ def test_phases(q, group, Ns, Nt, flux, flux8, kind):
         assert err.max() < 1e-10, (step, parity, mu, err.max())
     assert lat.exhausted == orc.exhausted
     lat.close()
+
+
+@pytest.mark.parametrize("kind", ["unitary", "scaled"])
+@pytest.mark.parametrize("Ns,Nt,flux,flux8", [(6, 2, 1, 0), (18, 4, 1, 1), (20, 4, 0, 0)])
+def test_su3_working_sweep_measurement(q, Ns, Nt, flux, flux8, kind):
+    """The plaquette sums on the last pass and the Polyakov loop in fixed point:
+    the links of the same sweep without them, and the numbers of the separate
+    measurement on those links (FP64 sums of 10^4 to 10^5 terms of order 1)."""
+    a = q.Lattice(3, Ns, Nt, 5.7, flux, FP64_PLAIN, HOT, 7, flux8=flux8)
+    b = q.Lattice(3, Ns, Nt, 5.7, flux, FP64_PLAIN, HOT, 7, flux8=flux8)
+    start = links_of(kind, a.get_links(), np.random.default_rng(3))
+    a.set_links(start)
+    b.set_links(start)
+    got = np.array(q.qcd_working_sweep(a.h, 1, 1, 5))
+    b.sweep(1, 1, 5)
+    assert np.array_equal(a.get_links(), b.get_links())
+    p, l = b.measure()
+    assert np.abs(got - np.array(p + l)).max() < 1e-13
+    a.close()
+    b.close()

@@ -18,7 +18,7 @@ pytestmark = pytest.mark.gpu
     (4, 1, 0.3, 1.0, 0.8, 1.0), (1, 6, 0.2, 0.5, 1.5, 1.0), (3, 131, 0.3, 1.0, 0.8, 1.0), (2, 300, 0.25, 2.0, 0.5, 1.0),
     (4, 7, 0.3, 1e6, 1e-3, 1.0),     # a stiff constraint: the bound is loose
     (2, 5, -0.3, -1e-9, 0.8, 1.0),   # signs turned
-    (4, 9, 0.3, 0.0, 1e30, 1e45),    # beyond FP32: every test in FP64
+    (4, 9, 0.3, 0.0, 1e45, 1e45),    # beyond FP32: every test in FP64
 ])
 def test_fp64_hits(N, nhit, kappa, lam, delta, scale):
     torch = pytest.importorskip("torch")
