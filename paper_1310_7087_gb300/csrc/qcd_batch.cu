@@ -57,7 +57,6 @@ struct BatchArgs {
   int stall_lattice;    // test hook: this lattice's barriers wait for one arrival too many (-1: off)
 };
 
-constexpr int BATCH_MAX_THREADS = 512;
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
   unsigned v;
@@ -99,28 +98,6 @@ __device__ bool group_barrier(const BatchArgs& b, int li, unsigned target) {
   }
   __syncthreads();
   return ok != 0;
-}
-
-__device__ __forceinline__ void block_sum4(double v[4], double* out) {
-  __shared__ double sh[4][BATCH_MAX_THREADS / 32];
-#pragma unroll
-  for (int k = 0; k < 4; ++k)
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], off);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < 4; ++k) sh[k][warp] = v[k];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const int nw = (blockDim.x + 31) / 32;
-    for (int k = 0; k < 4; ++k) {
-      double s = 0.0;
-      for (int w = 0; w < nw; ++w) s += sh[k][w];
-      out[k] = s;
-    }
-  }
-  __syncthreads();
 }
 
 // A thread's sites h = first, first + stride, ... of one parity, walked by
@@ -167,26 +144,27 @@ __device__ inline int4 site_digits(const Geom& g, int r) {
 }
 
 template <typename R, bool FIELD, int KIND, int MU>
-__device__ __forceinline__ double batch_update(const Ctx& a, int p, const LexSite& x, uint32_t sweep) {
+__device__ __forceinline__ R batch_update(const Ctx& a, int p, const LexSite& x, uint32_t sweep) {
   if constexpr (sizeof(R) == 8) return su2d_update_at<FIELD, KIND, MU, true>(a, p, x, sweep);
-  else return double(su2c_update_at<R, FIELD, KIND, MU, true>(a, p, x, sweep));
+  else return su2c_update_at<R, FIELD, KIND, MU, true>(a, p, x, sweep);
 }
 
-// One phase over this CTA's share of the lattice; returns the sum of the
-// updates' plaquette terms (KIND_OR_MEAS) in FP64.
+// One phase over this CTA's share of the lattice; KIND_OR_MEAS adds the updates'
+// plaquette terms to *v.
 // The digits of 2 stride are the same for the whole CTA: they are read from
 // shared memory (d) instead of being held in registers.
 template <typename R, bool FIELD, int KIND>
-__device__ __forceinline__ double batch_phase(const Ctx& a, int p, int mu, int first, int stride, const int4* d,
-                                              uint32_t sweep) {
-  double v = 0.0;
+__device__ __forceinline__ void batch_phase(const Ctx& a, int p, int mu, int first, int stride, const int4* d,
+                                            uint32_t sweep, SumOf<R>* v = nullptr) {
   const int4 r0 = site_digits(a.g, 2 * first);  // once per phase: nothing held across phases
   SiteWalk w{r0.x, r0.y, r0.z, r0.w};
   switch (mu) {
 #define QCD_BATCH_MU(MU)                                                                          \
   case MU:                                                                                        \
-    for (int h = first; h < a.g.Vh; h += stride, w.step(a.g.Ns, *d))                                  \
-      v += batch_update<R, FIELD, KIND, MU>(a, p, w.site(p, h), sweep);                            \
+    for (int h = first; h < a.g.Vh; h += stride, w.step(a.g.Ns, *d)) {                            \
+      const R t = batch_update<R, FIELD, KIND, MU>(a, p, w.site(p, h), sweep);                    \
+      if (KIND == KIND_OR_MEAS) v->add(t);                                                        \
+    }                                                                                             \
     break;
     QCD_BATCH_MU(0)
     QCD_BATCH_MU(1)
@@ -194,7 +172,6 @@ __device__ __forceinline__ double batch_phase(const Ctx& a, int p, int mu, int f
     QCD_BATCH_MU(3)
 #undef QCD_BATCH_MU
   }
-  return v;
 }
 
 template <typename R, bool FIELD>
@@ -240,7 +217,7 @@ __device__ void batch_run(const BatchArgs& b, int li, const BatchLat& L, int j) 
         batch_phase<R, FIELD, KIND_HB>(a, p, mu, first, stride, &step_digits, sweep);
         if (!barrier()) return;
       }
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    SumOf<R> v[4];
     // the last OR pass reunitarizes the links it updates and its odd phases
     // mu = 1..3 sum the plaquettes of the planes (mu, nu < mu), each once
     for (int o = 0; o < b.n_or; ++o)
@@ -249,7 +226,7 @@ __device__ void batch_run(const BatchArgs& b, int li, const BatchLat& L, int j) 
           if (o < b.n_or - 1) {
             batch_phase<R, FIELD, KIND_OR>(a, p, mu, first, stride, &step_digits, sweep);
           } else if (p == 1 && mu >= 1) {
-            v[mu == 3 ? 1 : 0] += batch_phase<R, FIELD, KIND_OR_MEAS>(a, p, mu, first, stride, &step_digits, sweep);
+            batch_phase<R, FIELD, KIND_OR_MEAS>(a, p, mu, first, stride, &step_digits, sweep, &v[mu == 3 ? 1 : 0]);
           } else {
             batch_phase<R, FIELD, KIND_OR_REUNIT>(a, p, mu, first, stride, &step_digits, sweep);
           }
@@ -264,7 +241,7 @@ __device__ void batch_run(const BatchArgs& b, int li, const BatchLat& L, int j) 
       for (int64_t idx = first; idx < V; idx += stride) plaquette_site<P, FIELD, true>(a, idx, v[0], v[1]);
     }
     for (int64_t idx = first; idx < V3; idx += stride) polyakov_site<P, true>(a, idx, v[2], v[3]);
-    block_sum4(v, b.partials + 4 * int64_t(blockIdx.x));
+    block_sums(v, b.partials + 4 * int64_t(blockIdx.x));
     if (!barrier()) return;
     if (j == 0 && threadIdx.x == 0) {
       double t[4] = {0.0, 0.0, 0.0, 0.0};

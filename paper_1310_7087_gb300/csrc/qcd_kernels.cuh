@@ -729,19 +729,22 @@ __global__ void set_frozen_kernel(const Ctx a) {
   P::store(a.links, a.g, mu, parity_of(x), lex(a.g, x) >> 1, u);
 }
 
-// Sum of v over the block (any multiple of 32 threads), in a fixed order,
-// written by thread 0; every thread of the block must call it.  No FP64
-// arithmetic inside the warp (FP64 runs at a small fraction of the FP32 rate,
-// and five dependent FP64 adds per thread at the end of every CTA held its
-// warps): each shuffle level adds by Knuth's error-free TwoSum, t + e = s + s' exactly,
-// and carries the errors in c; lane 0 adds s + c in FP64.  The warp sum keeps
-// a relative error near 2^-48 (the rounding of c), as an FP64 sum of the
-// FP32 inputs would; the warps are then added in FP64.
-__device__ __forceinline__ void block_sum_f32(float v, double* out) {
-  __shared__ double sh[32];
-  float s = v, c = 0.f;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
+// ---------------------------------------------------------------------------
+// Sums.  FP64 runs at a small fraction of the FP32 rate (one FP64 add of a warp
+// takes 64 cycles, and so does a conversion), so FP32 terms are summed without it:
+// Knuth's error-free TwoSum, t + e = s + s' exactly, keeps the errors in c, and
+// s + c is formed in FP64 once per warp.  The sum keeps a relative error near
+// 2^-48 (the rounding of c), as an FP64 sum of the FP32 terms would.
+// ---------------------------------------------------------------------------
+struct SumF {
+  float s = 0.f, c = 0.f;
+  __device__ __forceinline__ void add(float v) {
+    const float t = s + v;
+    const float bp = t - s;
+    c += (s - (t - bp)) + (v - bp);
+    s = t;
+  }
+  __device__ __forceinline__ void merge_down(int off) {
     const float so = __shfl_down_sync(0xffffffffu, s, off), co = __shfl_down_sync(0xffffffffu, c, off);
     const float t = s + so;
     const float bp = t - s;
@@ -749,49 +752,63 @@ __device__ __forceinline__ void block_sum_f32(float v, double* out) {
     s = t;
     c += co + e;
   }
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = double(s) + double(c);
+  __device__ __forceinline__ double value() const { return double(s) + double(c); }
+};
+struct SumD {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double v) { s += v; }
+  __device__ __forceinline__ void merge_down(int off) { s += __shfl_down_sync(0xffffffffu, s, off); }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <typename R>
+struct SumOfT {
+  using type = SumD;
+};
+template <>
+struct SumOfT<float> {
+  using type = SumF;
+};
+template <typename R>
+using SumOf = typename SumOfT<R>::type;
+
+// Sums of N values over the block (any multiple of 32 threads), in a fixed order,
+// written by N threads; every thread of the block must call it.
+template <int N, class Sum>
+__device__ __forceinline__ void block_sums(Sum (&v)[N], double* out) {
+  __shared__ double sh[N][32];
+#pragma unroll
+  for (int k = 0; k < N; ++k)
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v[k].merge_down(off);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane == 0)
+#pragma unroll
+    for (int k = 0; k < N; ++k) sh[k][warp] = v[k].value();
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double r = 0.0;
-    for (int w = 0; w < int(blockDim.x >> 5); ++w) r += sh[w];
-    *out = r;
+  if (threadIdx.x < N) {
+    double r = sh[threadIdx.x][0];
+    for (int w = 1; w < int(blockDim.x >> 5); ++w) r += sh[threadIdx.x][w];
+    out[threadIdx.x] = r;
   }
+}
+
+__device__ __forceinline__ void block_sum_f32(float v, double* out) {
+  SumF s[1];
+  s[0].s = v;
+  block_sums(s, out);
 }
 
 // ---------------------------------------------------------------------------
 // Measurements: plaquette (spatial / temporal split) and Polyakov loop.
-// Products in the storage precision, sums in FP64: per-thread value, warp
+// Products in the storage precision, sums as above: per-thread value, warp
 // shuffle, per-block partial, then one block sums the partials in a fixed
 // order (deterministic for a given lattice).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void block_sum2(double& v0, double& v1, double* partial_out) {
-  __shared__ double sh[2][MEAS_THREADS / 32];
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    v0 += __shfl_down_sync(0xffffffffu, v0, off);
-    v1 += __shfl_down_sync(0xffffffffu, v1, off);
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) {
-    sh[0][warp] = v0;
-    sh[1][warp] = v1;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s0 = 0.0, s1 = 0.0;
-    for (int w = 0; w < MEAS_THREADS / 32; ++w) {
-      s0 += sh[0][w];
-      s1 += sh[1][w];
-    }
-    partial_out[0] = s0;
-    partial_out[1] = s1;
-  }
-}
 
 // Plaquettes of one site (index idx over both parities): spatial sum into v0,
-// temporal sum into v1, (1/N) Re Tr each, FP64.
-template <class P, int FIELD, bool CG = false>
-__device__ __forceinline__ void plaquette_site(const Ctx& a, int64_t idx, double& v0, double& v1) {
+// temporal sum into v1, (1/N) Re Tr each.
+template <class P, int FIELD, bool CG = false, class Sum>
+__device__ __forceinline__ void plaquette_site(const Ctx& a, int64_t idx, Sum& v0, Sum& v1) {
   using R = typename P::Real;
   using A = Alg<R>;
   const int par = int(idx / a.g.Vh), h = int(idx % a.g.Vh);
@@ -805,16 +822,17 @@ __device__ __forceinline__ void plaquette_site(const Ctx& a, int64_t idx, double
       const Site xpn = step(a.g, x, nu, +1);
       const auto ab = A::mul(umu, load_eff<P, FIELD, CG>(a, nu, xpm));
       const auto dc = A::mul(load_eff<P, FIELD, CG>(a, nu, x), load_eff<P, FIELD, CG>(a, mu, xpn));
-      const double p = double(A::retr_nd_over_n(ab, dc));
-      if (nu == 3) v1 += p;
-      else v0 += p;
+      const R p = A::retr_nd_over_n(ab, dc);
+      if (nu == 3) v1.add(p);
+      else v0.add(p);
     }
   }
 }
 
-// Polyakov loop of spatial site idx: (1/N) Tr of the ordered t-product, FP64.
-template <class P, bool CG = false>
-__device__ __forceinline__ void polyakov_site(const Ctx& a, int64_t idx, double& v0, double& v1) {
+// Polyakov loop of spatial site idx: Tr of the ordered t-product (SU(2): half of
+// it); the final sums take the 1/3 of SU(3).
+template <class P, bool CG = false, class Sum>
+__device__ __forceinline__ void polyakov_site(const Ctx& a, int64_t idx, Sum& v0, Sum& v1) {
   using R = typename P::Real;
   using A = Alg<R>;
   Site x;
@@ -828,135 +846,111 @@ __device__ __forceinline__ void polyakov_site(const Ctx& a, int64_t idx, double&
     l = A::mul(l, P::template load<CG>(a.links, a.g, 3, parity_of(x), lex(a.g, x) >> 1));
   }
   if constexpr (P::N == 2) {
-    v0 += double(l.q0);
+    v0.add(l.q0);
   } else {
-    v0 += (double(l.e[0][0].re) + double(l.e[1][1].re) + double(l.e[2][2].re)) / 3.0;
-    v1 += (double(l.e[0][0].im) + double(l.e[1][1].im) + double(l.e[2][2].im)) / 3.0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      v0.add(l.e[k][k].re);
+      v1.add(l.e[k][k].im);
+    }
   }
 }
 
 template <class P, int FIELD>
 __global__ void __launch_bounds__(MEAS_THREADS, 2) measure_kernel(const Ctx a, int n_plaq_blocks) {
-  double v0 = 0.0, v1 = 0.0;
+  SumOf<typename P::Real> v[2];
   if (int(blockIdx.x) < n_plaq_blocks) {
     const int64_t idx = int64_t(blockIdx.x) * MEAS_THREADS + threadIdx.x;
-    if (idx < 2LL * a.g.Vh) plaquette_site<P, FIELD>(a, idx, v0, v1);
+    if (idx < 2LL * a.g.Vh) plaquette_site<P, FIELD>(a, idx, v[0], v[1]);
   } else {
     const int64_t idx = int64_t(int(blockIdx.x) - n_plaq_blocks) * MEAS_THREADS + threadIdx.x;
-    if (idx < int64_t(a.g.Ns) * a.g.Ns * a.g.Ns) polyakov_site<P>(a, idx, v0, v1);
+    if (idx < int64_t(a.g.Ns) * a.g.Ns * a.g.Ns) polyakov_site<P>(a, idx, v[0], v[1]);
   }
-  block_sum2(v0, v1, a.partials + 2 * blockIdx.x);
+  block_sums(v, a.partials + 2 * blockIdx.x);
 }
 
-// Sums the per-block partials in a fixed order and normalises:
-// out = {P, P_s, P_t, Re L, Im L}.
-static __global__ void __launch_bounds__(FINAL_THREADS)
-    measure_final_kernel(const Ctx a, int n_plaq_blocks, int n_poly_blocks) {
-  __shared__ double sh[4][FINAL_THREADS];
-  double s[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int b = threadIdx.x; b < n_plaq_blocks; b += FINAL_THREADS) {
-    s[0] += a.partials[2 * b];
-    s[1] += a.partials[2 * b + 1];
-  }
-  for (int b = threadIdx.x; b < n_poly_blocks; b += FINAL_THREADS) {
-    s[2] += a.partials[2 * (n_plaq_blocks + b)];
-    s[3] += a.partials[2 * (n_plaq_blocks + b) + 1];
-  }
+// Final sums: one block whose warps share N series of block partials, series k at
+// p + offset[k] with n[k] entries `stride[k]` apart; W warps per series, blockDim =
+// 32 N W.  Only as many warps as the series fill: the 25 FP64 adds of a warp's
+// shuffles at 64 cycles each were most of the kernel when 32 warps did them (working
+// sweep of SU(2) FP32 4^3x4 with its tail 61.4 -> 49.2 us, SU(3) FP32 16^3x4 270 ->
+// 258).  Returns the sums in sh[k][0] to every thread.
+template <int N>
+__device__ __forceinline__ void final_sums(const double* const (&p)[N], const int (&n)[N], const int (&stride)[N],
+                                           double (&sh)[N][8]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = int(blockDim.x >> 5) / N;
+  const int k = warp % N, w = warp / N;
+  double s = 0.0;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) sh[k][threadIdx.x] = s[k];
-  __syncthreads();
-  for (int w = FINAL_THREADS / 2; w > 0; w >>= 1) {
-    if (int(threadIdx.x) < w) {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) sh[k][threadIdx.x] += sh[k][threadIdx.x + w];
+  for (int q = 0; q < N; ++q)
+    if (q == k) {
+      double s2 = 0.0;
+      int b = 32 * w + lane;
+      for (; b + 32 * W < n[q]; b += 64 * W) {
+        const double x = p[q][int64_t(b) * stride[q]], y = p[q][int64_t(b + 32 * W) * stride[q]];
+        s += x;
+        s2 += y;
+      }
+      if (b < n[q]) s += p[q][int64_t(b) * stride[q]];
+      if (n[q] > 32 * W) s += s2;
     }
-    __syncthreads();
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+  if (lane == 0) sh[k][w] = s;
+  __syncthreads();
+  if (threadIdx.x < N) {
+    double r = sh[threadIdx.x][0];
+    for (int v = 1; v < W; ++v) r += sh[threadIdx.x][v];
+    sh[threadIdx.x][0] = r;
   }
-  if (threadIdx.x == 0) {
-    const double V = 2.0 * double(a.g.Vh);
-    const double V3 = double(a.g.Ns) * a.g.Ns * a.g.Ns;
-    a.meas_out[0] = (sh[0][0] + sh[1][0]) / (6.0 * V);
-    a.meas_out[1] = sh[0][0] / (3.0 * V);
-    a.meas_out[2] = sh[1][0] / (3.0 * V);
-    a.meas_out[3] = sh[2][0] / V3;
-    a.meas_out[4] = sh[3][0] / V3;
+  __syncthreads();
+}
+// Warps per series for the longest series' length.
+inline int final_warps(int n) { return std::max(1, std::min(6, (n + 127) / 128)); }
+
+// out = {P, P_s, P_t, Re L, Im L} of the measurement's block partials; one thread
+// per number (one FP64 division each).
+static __global__ void __launch_bounds__(FINAL_THREADS)
+    measure_final_kernel(const Ctx a, int n_plaq_blocks, int n_poly_blocks, double poly_scale) {
+  __shared__ double sh[4][8];
+  const double* q = a.partials + 2 * int64_t(n_plaq_blocks);
+  final_sums<4>({a.partials, a.partials + 1, q, q + 1}, {n_plaq_blocks, n_plaq_blocks, n_poly_blocks, n_poly_blocks},
+                {2, 2, 2, 2}, sh);
+  if (threadIdx.x < 5) {
+    const double V = 2.0 * double(a.g.Vh), V3 = double(a.g.Ns) * a.g.Ns * a.g.Ns;
+    const int t = threadIdx.x;
+    const double num = t == 0 ? sh[0][0] + sh[1][0] : t < 3 ? sh[t - 1][0] : sh[t - 1][0] * poly_scale;
+    a.meas_out[t] = num / (t == 0 ? 6.0 * V : t < 3 ? 3.0 * V : V3);
   }
 }
 
 // Final sums of a working sweep's fused measurement: the plaquette partials
 // of the three plane-summing phases of the last pass (odd parity, mu = 1, 2,
-// 3; `grid` block partials each) and the Polyakov-loop partials.  Writes
-// meas_out = {P, P_s, P_t, Re L, Im L, P_1, P_2, P_3}, P_mu the mean plaquette
-// of the planes phase mu sums: (y,x); (z,x), (z,y); (t,x), (t,y), (t,z).
-// Two strided steps per loop keep six loads of the one block in flight; the
-// per-thread sums are reduced by warp shuffles and then across the 32 warps,
-// all in a fixed order.
-// plane_scale multiplies the plane sums: 1 when the phase kernels summed
-// (1/N) Re Tr, 1/N when they summed Re Tr.  The Polyakov loop's nl block partials
-// lie at poly_offset.
+// 3; `grid` block partials each) and the Polyakov-loop partials (nl pairs at
+// poly_offset).  Writes meas_out = {P, P_s, P_t, Re L, Im L, P_1, P_2, P_3}, P_mu the
+// mean plaquette of the planes phase mu sums: (y,x); (z,x), (z,y); (t,x), (t,y),
+// (t,z).  plane_scale multiplies the plane sums: 1 when the phase kernels summed
+// (1/N) Re Tr, 1/N when they summed Re Tr; poly_scale the Polyakov loop.
 static __global__ void __launch_bounds__(FINAL_THREADS)
-    fused_final_kernel(const Ctx a, int grid, double plane_scale, int nl, int poly_offset) {
-  constexpr int NW = FINAL_THREADS / 32;
-  __shared__ double sh[5][NW];
+    fused_final_kernel(const Ctx a, int grid, double plane_scale, int nl, int poly_offset, double poly_scale) {
+  __shared__ double sh[5][8];
   const double* pl = a.partials + poly_offset;
-  const double* p1 = a.partials + fused_plaq_offset(a.g, 1);
-  const double* p2 = a.partials + fused_plaq_offset(a.g, 2);
-  const double* p3 = a.partials + fused_plaq_offset(a.g, 3);
-  double s[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  int b = threadIdx.x;
-  for (; b + FINAL_THREADS < grid; b += 2 * FINAL_THREADS) {
-    const double x1 = p1[b], x2 = p2[b], x3 = p3[b];
-    const double y1 = p1[b + FINAL_THREADS], y2 = p2[b + FINAL_THREADS], y3 = p3[b + FINAL_THREADS];
-    s[0] += x1;
-    s[1] += x2;
-    s[2] += x3;
-    s[0] += y1;
-    s[1] += y2;
-    s[2] += y3;
+  final_sums<5>({a.partials + fused_plaq_offset(a.g, 1), a.partials + fused_plaq_offset(a.g, 2),
+                 a.partials + fused_plaq_offset(a.g, 3), pl, pl + 1},
+                {grid, grid, grid, nl, nl}, {1, 1, 1, 2, 2}, sh);
+  if (threadIdx.x < 8) {
+    const double V = 2.0 * double(a.g.Vh), V3 = double(a.g.Ns) * a.g.Ns * a.g.Ns;
+    const int t = threadIdx.x;
+    const double sp = sh[0][0] + sh[1][0];
+    const double num = t == 0 ? sp + sh[2][0] : t == 1 ? sp : t == 2 ? sh[2][0] : t < 5 ? sh[t][0] : sh[t - 5][0];
+    const double den = t == 0 ? 6.0 * V : t < 3 || t == 7 ? 3.0 * V : t < 5 ? V3 : t == 5 ? V : 2.0 * V;
+    a.meas_out[t] = num * (t == 3 || t == 4 ? poly_scale : plane_scale) / den;
   }
-  for (; b < grid; b += FINAL_THREADS) {
-    s[0] += p1[b];
-    s[1] += p2[b];
-    s[2] += p3[b];
-  }
-  for (int c = threadIdx.x; c < nl; c += FINAL_THREADS) {
-    s[3] += pl[2 * c];
-    s[4] += pl[2 * c + 1];
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < 5; ++k) {
-    double v = s[k];
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    if (lane == 0) sh[k][warp] = v;
-  }
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      double v = lane < NW ? sh[k][lane] : 0.0;
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-      s[k] = v;
-    }
-    if (lane == 0) {
-      const double V = 2.0 * double(a.g.Vh);
-      const double V3 = double(a.g.Ns) * a.g.Ns * a.g.Ns;
-      s[0] *= plane_scale;
-      s[1] *= plane_scale;
-      s[2] *= plane_scale;
-      const double sp = s[0] + s[1];
-      a.meas_out[0] = (sp + s[2]) / (6.0 * V);
-      a.meas_out[1] = sp / (3.0 * V);
-      a.meas_out[2] = s[2] / (3.0 * V);
-      a.meas_out[3] = s[3] / V3;
-      a.meas_out[4] = s[4] / V3;
-      a.meas_out[5] = s[0] / V;
-      a.meas_out[6] = s[1] / (2.0 * V);
-      a.meas_out[7] = s[2] / (3.0 * V);
-    }
-  }
+}
+inline void launch_fused_final(const Ctx& a, cudaStream_t st, int grid, double plane_scale, int nl, int poly_offset,
+                               double poly_scale) {
+  const int block = 32 * 5 * final_warps(std::max(grid, nl));
+  fused_final_kernel<<<1, block, 0, st>>>(a, grid, plane_scale, nl, poly_offset, poly_scale);
 }
 
 // ---------------------------------------------------------------------------
@@ -1065,7 +1059,7 @@ cudaError_t launch_measure(const Ctx& a, int effective, cudaStream_t st) {
       default: measure_kernel<P, 2><<<np + nl, MEAS_THREADS, 0, st>>>(a, np); break;
     }
   }
-  measure_final_kernel<<<1, FINAL_THREADS, 0, st>>>(a, np, nl);
+  measure_final_kernel<<<1, 32 * 4 * final_warps(std::max(np, nl)), 0, st>>>(a, np, nl, P::N == 3 ? 1.0 / 3.0 : 1.0);
   return cudaGetLastError();
 }
 

@@ -157,20 +157,6 @@ __global__ void su2c_phase_kernel(const Ctx a, int parity) {
   su2c_update<R, FIELD, KIND, MU, false>(a, parity, h, KIND == KIND_HB ? *a.sweep : 0u);
 }
 
-// Sum of v over the block (any multiple of 32 threads) in a fixed order.
-__device__ __forceinline__ void su2c_block_sum(double v, double* out) {
-  __shared__ double sh[32];
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int w = 0; w < int(blockDim.x >> 5); ++w) s += sh[w];
-    *out = s;
-  }
-}
-
 // Last-pass phase (odd parity, MU >= 1) of a working sweep: update,
 // reunitarize and sum the plaquettes of the planes (MU, nu < MU).
 template <typename R, bool FIELD, int MU>
@@ -178,15 +164,14 @@ __global__ void su2c_or_meas_kernel(const Ctx a, int parity) {
   const int h = blockIdx.x * blockDim.x + threadIdx.x;
   R v = R(0);
   if (h < a.g.Vh) v = su2c_update<R, FIELD, KIND_OR_MEAS, MU, false>(a, parity, h, 0u);
-  if constexpr (sizeof(R) == 4) block_sum_f32(v, a.partials + fused_plaq_offset(a.g, MU) + blockIdx.x);
-  else su2c_block_sum(v, a.partials + fused_plaq_offset(a.g, MU) + blockIdx.x);
+  block_sum_f32(v, a.partials + fused_plaq_offset(a.g, MU) + blockIdx.x);
 }
 
 template <typename R>
 cudaError_t su2c_measure_fused_tail(const Ctx& a, int block, cudaStream_t st) {
   const int nl = meas_poly_blocks(a.g);
   measure_kernel<SU2Policy<R>, 0><<<nl, MEAS_THREADS, 0, st>>>(a, 0);  // Polyakov loop only
-  fused_final_kernel<<<1, FINAL_THREADS, 0, st>>>(a, int(grid_for(a.g.Vh, block)), 1.0, nl, 0);
+  launch_fused_final(a, st, int(grid_for(a.g.Vh, block)), 1.0, nl, 0, 1.0);
   return cudaGetLastError();
 }
 

@@ -281,7 +281,9 @@ __global__ void __maxnreg__(128) su2d_phase_kernel(const __grid_constant__ Ctx a
   if (KIND == KIND_OR_MEAS) {
     double* out = a.partials + fused_plaq_offset(a.g, MU) + blockIdx.x;
     if (SPLIT == 1) {
-      su2c_block_sum(v, out);
+      SumD s[1];
+      s[0].s = v;
+      block_sums(s, out);
     } else {  // one warp is left
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);

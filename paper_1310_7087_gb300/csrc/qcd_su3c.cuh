@@ -491,18 +491,18 @@ __global__ void __maxnreg__(QCD_SU3_MEAS_MAXNREG) su3c_or_meas_kernel(const Ctx 
   block_sum_f32(v, a.partials + fused_plaq_offset(a.g, MU) + blockIdx.x);
 }
 
-// Polyakov loop of a working sweep's fused measurement: (1/3) Tr of the
+// Polyakov loop of a working sweep's fused measurement: Tr of the
 // ordered product over t of the t-links of each spatial site, one thread per
 // site, products formed by rows 0-1 with row 2 rebuilt as for every FP32 link
 // (with the final-sum kernel below: measurement tail 0.107 -> 0.077 ms per
 // working sweep at 64^3x16, against the generic full-matrix product;
 // splitting each product over 2 or 4 lanes with a shuffle tree measured
 // slower, 0.094 / 0.127 ms, and so did unrolling the t-loop by 4, 0.091 ms).
-// Block partials of Re and Im, FP64, in a fixed order.
+// Block partials of Re and Im in a fixed order.
 static __global__ void __launch_bounds__(MEAS_THREADS) su3c_poly_kernel(const Ctx a) {
   const long long V3 = (long long)a.g.Ns * a.g.Ns * a.g.Ns;
   const long long site = (long long)blockIdx.x * MEAS_THREADS + threadIdx.x;
-  double v0 = 0.0, v1 = 0.0;
+  SumF v[2];
   if (site < V3) {
     const int Ns = a.g.Ns;
     const int x = int(site % Ns), y = int((site / Ns) % Ns), z = int(site / ((long long)Ns * Ns));
@@ -512,15 +512,19 @@ static __global__ void __launch_bounds__(MEAS_THREADS) su3c_poly_kernel(const Ct
     for (int t = 1; t < a.g.Nt; ++t)
       l = su3c_mul(l, su3c_full(su3c_load(a.links, a.g, 3, (xyz + t) & 1, int((s0 + (long long)t * V3) >> 1))));
     const Cx<float> l22 = cross2(l.e[0][0], l.e[1][1], l.e[0][1], l.e[1][0]);
-    v0 = (double(l.e[0][0].re) + double(l.e[1][1].re) + double(l22.re)) / 3.0;
-    v1 = (double(l.e[0][0].im) + double(l.e[1][1].im) + double(l22.im)) / 3.0;
+    v[0].add(l.e[0][0].re);
+    v[0].add(l.e[1][1].re);
+    v[0].add(l22.re);
+    v[1].add(l.e[0][0].im);
+    v[1].add(l.e[1][1].im);
+    v[1].add(l22.im);
   }
-  block_sum2(v0, v1, a.partials + 2 * blockIdx.x);
+  block_sums(v, a.partials + 2 * blockIdx.x);
 }
 
 inline cudaError_t su3c_measure_fused_tail(const Ctx& a, int block, cudaStream_t st) {
   su3c_poly_kernel<<<meas_poly_blocks(a.g), MEAS_THREADS, 0, st>>>(a);
-  fused_final_kernel<<<1, FINAL_THREADS, 0, st>>>(a, int(grid_for(a.g.Vh, block)), 1.0 / 3.0, meas_poly_blocks(a.g), 0);
+  launch_fused_final(a, st, int(grid_for(a.g.Vh, block)), 1.0 / 3.0, meas_poly_blocks(a.g), 0, 1.0 / 3.0);
   return cudaGetLastError();
 }
 

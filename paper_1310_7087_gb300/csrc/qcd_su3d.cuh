@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(96 * SPLIT, SU3D_CTAS / SPLIT)
 
 // Polyakov loop of a working sweep's fused measurement: three warps per 32 spatial
 // sites, warp r with row r of the running product over t; each converts row r of
-// the next link for the three.  FP64 block partials of (1/3) Tr, in a fixed order.
+// the next link for the three.  FP64 block partials of Tr, in a fixed order.
 // (The plane sums, this kernel and the final sums add 41 us to a sweep of 16^3x4 and
 // 77 to one of 32^3x8; the separate FP64 measurement took 128 and 780.)
 static __global__ void __launch_bounds__(96) su3d_poly_kernel(const __grid_constant__ Ctx a) {
@@ -490,15 +490,15 @@ static __global__ void __launch_bounds__(96) su3d_poly_kernel(const __grid_const
   const bool fixed = in && !out_of_range;
   double re = fx_warp_sum(fixed ? fx_value(d.re) : 0), im = fx_warp_sum(fixed ? fx_value(d.im) : 0);
   if (role == 0 && __any_sync(0xffffffffu, in && out_of_range)) {
-    double v0 = 0.0, v1 = 0.0;
+    SumD v0, v1;
     if (in && out_of_range) polyakov_site<SU3Policy<double>>(a, site, v0, v1);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
-      v0 += __shfl_down_sync(0xffffffffu, v0, off);
-      v1 += __shfl_down_sync(0xffffffffu, v1, off);
+      v0.merge_down(off);
+      v1.merge_down(off);
     }
-    re += 3.0 * v0;
-    im += 3.0 * v1;
+    re += v0.s;
+    im += v1.s;
   }
   if (lane == 0) {
     sum[role][0] = re;
@@ -507,13 +507,13 @@ static __global__ void __launch_bounds__(96) su3d_poly_kernel(const __grid_const
   __syncthreads();
   if (threadIdx.x < 2)
     a.partials[fused_plaq_offset(a.g, 4) + 2 * blockIdx.x + threadIdx.x] =
-        (sum[0][threadIdx.x] + sum[1][threadIdx.x] + sum[2][threadIdx.x]) / 3.0;
+        sum[0][threadIdx.x] + sum[1][threadIdx.x] + sum[2][threadIdx.x];
 }
 
 inline cudaError_t su3d_measure_fused_tail(const Ctx& a, int /*block*/, cudaStream_t st) {
   const int nl = fused_poly32_blocks(a.g);
   su3d_poly_kernel<<<nl, 96, 0, st>>>(a);
-  fused_final_kernel<<<1, FINAL_THREADS, 0, st>>>(a, (a.g.Vh + 31) / 32, 1.0 / 3.0, nl, fused_plaq_offset(a.g, 4));
+  launch_fused_final(a, st, (a.g.Vh + 31) / 32, 1.0 / 3.0, nl, fused_plaq_offset(a.g, 4), 1.0 / 3.0);
   return cudaGetLastError();
 }
 
