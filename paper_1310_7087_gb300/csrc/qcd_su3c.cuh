@@ -23,8 +23,6 @@
 
 #include "qcd_kernels.cuh"
 
-
-
 namespace qcd {
 
 // Rows 0 and 1 of an SU(3) matrix.
@@ -243,6 +241,24 @@ __device__ __forceinline__ void su3c_conj_row2(M3<float>& m) {
   for (int c = 0; c < 3; ++c) m.e[2][c].im = -m.e[2][c].im;
 }
 
+// Rows 0-1 of one staple of U_MU(x), x of parity p: the upper one,
+// Ut_nu(x+mu) Ut_mu(x+nu)^+ Ut_nu(x)^+, or the lower one,
+// (Ut_mu(x-nu) Ut_nu(x+mu-nu))^+ Ut_nu(x-nu).
+template <int FIELD, int MU, int NU, bool LOWER>
+__device__ __forceinline__ Rows2 su3c_one_staple(const Ctx& a, int p, const LexSite& x, const LexSite& xp) {
+  if (!LOWER) {
+    const LexSite xpn = lex_step<NU, +1>(a.g, x);
+    const Rows2 x1 = su3c_mul_nd(su3c_eff<FIELD, NU>(a, p ^ 1, xp), su3c_full(su3c_eff<FIELD, MU>(a, p ^ 1, xpn)));
+    return su3c_mul_nd(x1, su3c_full(su3c_eff<FIELD, NU>(a, p, x)));
+  } else {
+    const LexSite xmn = lex_step<NU, -1>(a.g, x);
+    const LexSite xpmn = lex_step<NU, -1>(a.g, xp);
+    const M3<float> y =
+        su3c_full(su3c_mul(su3c_eff<FIELD, MU>(a, p ^ 1, xmn), su3c_full(su3c_eff<FIELD, NU>(a, p, xpmn))));
+    return su3c_mul_dn(y, su3c_full(su3c_eff<FIELD, NU>(a, p ^ 1, xmn)));
+  }
+}
+
 // Staple sum of U_MU(x) (x of parity p) on effective links, full 3x3 (row 2
 // accumulated conjugated, see su3c_acc_c).
 // With SPLIT, *low receives the part of the sum over nu < MU.
@@ -262,21 +278,11 @@ __device__ __forceinline__ M3<float> su3c_staple(const Ctx& a, int p, const LexS
     }
     // Each branch of this switch is one static value of NU.
     switch (nu) {
-#define QCD_SU3C_NU(NU)                                                                         \
-  case NU: {                                                                                      \
-    const LexSite xpn = lex_step<NU, +1>(a.g, x);                                                \
-    const LexSite xmn = lex_step<NU, -1>(a.g, x);                                                \
-    const LexSite xpmn = lex_step<NU, -1>(a.g, xp);                                              \
-    /* upper: Ut_nu(x+mu) Ut_mu(x+nu)^+ Ut_nu(x)^+ */                                             \
-    const Rows2 x1 = su3c_mul_nd(su3c_eff<FIELD, NU>(a, p ^ 1, xp),                               \
-                                 su3c_full(su3c_eff<FIELD, MU>(a, p ^ 1, xpn)));                  \
-    su3c_acc_c(A, su3c_mul_nd(x1, su3c_full(su3c_eff<FIELD, NU>(a, p, x))));                      \
-    /* lower: (Ut_mu(x-nu) Ut_nu(x+mu-nu))^+ Ut_nu(x-nu) */                                      \
-    const M3<float> y = su3c_full(su3c_mul(su3c_eff<FIELD, MU>(a, p ^ 1, xmn),                   \
-                                           su3c_full(su3c_eff<FIELD, NU>(a, p, xpmn))));          \
-    su3c_acc_c(A, su3c_mul_dn(y, su3c_full(su3c_eff<FIELD, NU>(a, p ^ 1, xmn))));                 \
-    break;                                                                                        \
-  }
+#define QCD_SU3C_NU(NU)                                            \
+  case NU:                                                         \
+    su3c_acc_c(A, su3c_one_staple<FIELD, MU, NU, false>(a, p, x, xp)); \
+    su3c_acc_c(A, su3c_one_staple<FIELD, MU, NU, true>(a, p, x, xp));  \
+    break;
       QCD_SU3C_NU(0)
       QCD_SU3C_NU(1)
       QCD_SU3C_NU(2)
@@ -456,6 +462,29 @@ __global__ void __maxnreg__(KIND == KIND_HB          ? QCD_SU3_HB_MAXNREG
 #define QCD_SU3_MEAS_MAXNREG 128
 #endif
 
+// Re Tr(Ut low) of an updated link (the final sums take the 1/3).
+template <int FIELD, int MU>
+__device__ __forceinline__ float su3c_plane_sum(const Ctx& a, const LexSite& x, M3<float> U, const M3<float>& low) {
+  su3c_rebuild(U);  // row 2 as every later load rebuilds it
+  if (FIELD == 1 && MU == 1) {
+    const float2 ph = __ldg(a.phase32 + x.c[0]);
+    const Cx<float> pp{ph.x, ph.y}, pc{ph.x, -ph.y};
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      U.e[r][0] = cmul_pm(U.e[r][0], pp);
+      U.e[r][1] = cmul_pm(U.e[r][1], pc);
+    }
+  } else if (FIELD == 2 && MU == 1) {
+    Cx<float> b[3];
+    load_bdiag<float>(a, x.c[0], b);
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) U.e[r][k] = cmul_pm(U.e[r][k], b[k]);
+  }
+  return m3_retrace_mul(U, low);
+}
+
 template <int FIELD, int MU>
 __global__ void __maxnreg__(QCD_SU3_MEAS_MAXNREG) su3c_or_meas_kernel(const Ctx a, int parity) {
   pdl_launch_dependents();
@@ -469,27 +498,111 @@ __global__ void __maxnreg__(QCD_SU3_MEAS_MAXNREG) su3c_or_meas_kernel(const Ctx 
     const M3<float> A = su3c_staple<FIELD, MU, true>(a, parity, x, &low);
     M3<float> U = su3c_update<FIELD, KIND_OR_MEAS, MU>(a, parity, h, x, A,
                                                        su3c_full(su3c_load(a.links, a.g, MU, parity, h)));
-    su3c_rebuild(U);  // row 2 as every later load rebuilds it
-    if (FIELD == 1 && MU == 1) {
-      const float2 ph = __ldg(a.phase32 + x.c[0]);
-      const Cx<float> pp{ph.x, ph.y}, pc{ph.x, -ph.y};
-#pragma unroll
-      for (int r = 0; r < 3; ++r) {
-        U.e[r][0] = cmul_pm(U.e[r][0], pp);
-        U.e[r][1] = cmul_pm(U.e[r][1], pc);
-      }
-    } else if (FIELD == 2 && MU == 1) {
-      Cx<float> b[3];
-      load_bdiag<float>(a, x.c[0], b);
-#pragma unroll
-      for (int r = 0; r < 3; ++r)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) U.e[r][k] = cmul_pm(U.e[r][k], b[k]);
-    }
-    v = m3_retrace_mul(U, low);  // Re Tr; the final sums take the 1/3
+    v = su3c_plane_sum<FIELD, MU>(a, x, U, low);
   }
   block_sum_f32(v, a.partials + fused_plaq_offset(a.g, MU) + blockIdx.x);
 }
+
+// Small lattices: six warps share 32 links (lane = link), each computes one staple;
+// warp 0 adds them up in the order of su3c_staple, so that the results are the
+// same to the bit, and updates the links.  The heat-bath's draws ahead are spread
+// over warps 3 to 5.
+struct Su3cSplitShared {
+  float4 t[6][3][32];
+  float first[3][6][32];
+};
+
+template <int FIELD, int KIND, int MU>
+__global__ void __launch_bounds__(192, 3) su3c_split_kernel(const Ctx a, int parity) {
+  pdl_launch_dependents();
+  __shared__ Su3cSplitShared sh;
+  const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
+  const int i = blockIdx.x * 32 + lane;
+  const bool in = i < a.g.Vh;
+  const LexSite x = lex_site_ytz(a.g, parity, in ? i : a.g.Vh - 1);
+  const bool on = in && !frozen_link(a, MU, x.c[3]);
+  const LexSite xp = lex_step<MU, +1>(a.g, x);
+  pdl_wait();
+  uint32_t sweep = 0;
+  if (KIND == KIND_HB) sweep = *a.sweep;
+  Rows2 own;
+  if (role == 0) own = su3c_load(a.links, a.g, MU, parity, x.s >> 1);
+  Rows2 t;
+  switch (role) {
+#define QCD_SU3C_ROLE(N)                                                                                  \
+  case 2 * N: t = su3c_one_staple<FIELD, MU, N + (N >= MU), false>(a, parity, x, xp); break;               \
+  case 2 * N + 1: t = su3c_one_staple<FIELD, MU, N + (N >= MU), true>(a, parity, x, xp); break;
+    QCD_SU3C_ROLE(0)
+    QCD_SU3C_ROLE(1)
+    QCD_SU3C_ROLE(2)
+#undef QCD_SU3C_ROLE
+  }
+  sh.t[role][0][lane] = make_float4(t.e[0][0].re, t.e[0][0].im, t.e[0][1].re, t.e[0][1].im);
+  sh.t[role][1][lane] = make_float4(t.e[0][2].re, t.e[0][2].im, t.e[1][0].re, t.e[1][0].im);
+  sh.t[role][2][lane] = make_float4(t.e[1][1].re, t.e[1][1].im, t.e[1][2].re, t.e[1][2].im);
+  if (KIND == KIND_HB && role >= 3) {
+    const int sub = role - 3;
+    const KpFirst f = su3c_kp_first(make_stream(a.k0, a.k1, uint32_t(x.s), sweep, MU, sub, KIND_TRY),
+                                    make_stream(a.k0, a.k1, uint32_t(x.s), sweep, MU, sub, KIND_DIR));
+    sh.first[sub][0][lane] = f.e;
+    sh.first[sub][1][lane] = f.a3;
+    sh.first[sub][2][lane] = f.st;
+    sh.first[sub][3][lane] = f.ct;
+    sh.first[sub][4][lane] = f.sp;
+    sh.first[sub][5][lane] = f.cp;
+  }
+  __syncthreads();
+  if (role > 0) return;
+  M3<float> A, low;
+  m3_zero(A);
+#pragma unroll
+  for (int s = 0; s < 6; ++s) {
+    if (KIND == KIND_OR_MEAS && s == 2 * MU) {
+      low = A;
+      su3c_conj_row2(low);
+    }
+    const float4 u = sh.t[s][0][lane], v = sh.t[s][1][lane], w = sh.t[s][2][lane];
+    Rows2 r;
+    r.e[0][0] = {u.x, u.y};
+    r.e[0][1] = {u.z, u.w};
+    r.e[0][2] = {v.x, v.y};
+    r.e[1][0] = {v.z, v.w};
+    r.e[1][1] = {w.x, w.y};
+    r.e[1][2] = {w.z, w.w};
+    su3c_acc_c(A, r);
+  }
+  if (KIND == KIND_OR_MEAS && MU == 3) {
+    low = A;
+    su3c_conj_row2(low);
+  }
+  su3c_conj_row2(A);
+  KpFirst first[3];
+  if (KIND == KIND_HB)
+#pragma unroll
+    for (int sub = 0; sub < 3; ++sub)
+      first[sub] = {sh.first[sub][0][lane], sh.first[sub][1][lane], sh.first[sub][2][lane],
+                    sh.first[sub][3][lane], sh.first[sub][4][lane], sh.first[sub][5][lane]};
+  SumF v;
+  if (on) {
+    M3<float> U = su3c_update<FIELD, KIND, MU>(a, parity, x.s >> 1, x, A, su3c_full(own), first, sweep);
+    if (KIND == KIND_OR_MEAS) v.s = su3c_plane_sum<FIELD, MU>(a, x, U, low);
+  }
+  if (KIND == KIND_OR_MEAS) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v.merge_down(off);
+    if (lane == 0) a.partials[fused_plaq_offset(a.g, MU) + blockIdx.x] = v.value();
+  }
+}
+
+// Split up to 800 CTAs of 32 links: sweeps of 1 heat-bath + 4 overrelaxation
+// passes, us, not split / split: 4^3x4 229 / 115, 12^3x4 (108 CTAs) 230 / 144, 16^3x4
+// (256) 240 / 159, 20^3x4 (500) 289 / 232, 20^3x6 (750) 288 / 255, 24^3x6 (1296) 326 /
+// 349.  At these sizes a phase is one chain of latencies (one warp per SM
+// sub-partition or less): the gather's loads, 12 products one after another, the
+// update; the split takes the products and most of the loads out of the chain.
+inline bool su3c_split(const GeomH& g) { return (g.Vh + 31) / 32 <= 800; }
+// Links of one CTA for a block size of the caller.
+inline int su3c_links_per_cta(const GeomH& g, int block) { return su3c_split(g) ? 32 : block; }
 
 // Polyakov loop of a working sweep's fused measurement: Tr of the
 // ordered product over t of the t-links of each spatial site, one thread per
@@ -524,7 +637,8 @@ static __global__ void __launch_bounds__(MEAS_THREADS) su3c_poly_kernel(const Ct
 
 inline cudaError_t su3c_measure_fused_tail(const Ctx& a, int block, cudaStream_t st) {
   su3c_poly_kernel<<<meas_poly_blocks(a.g), MEAS_THREADS, 0, st>>>(a);
-  launch_fused_final(a, st, int(grid_for(a.g.Vh, block)), 1.0 / 3.0, meas_poly_blocks(a.g), 0, 1.0 / 3.0);
+  launch_fused_final(a, st, int(grid_for(a.g.Vh, su3c_links_per_cta(a.g, block))), 1.0 / 3.0, meas_poly_blocks(a.g), 0,
+                     1.0 / 3.0);
   return cudaGetLastError();
 }
 
@@ -548,7 +662,18 @@ inline void launch_programmatic(void (*kernel)(P...), unsigned grid, int block, 
 }
 
 template <int FIELD, int KIND, int MU>
+inline void su3c_launch_split(const Ctx& a, int parity, cudaStream_t st) {
+  // Programmatic launch beyond one wave of 3 CTAs per SM (20^3x4: 246 -> 232 us per
+  // sweep); within one it places the next phase's CTAs on the SMs that are left
+  // (4^3x4: 115 -> 136).
+  const unsigned grid = grid_for(a.g.Vh, 32);
+  if (grid > 3 * 152) launch_programmatic(su3c_split_kernel<FIELD, KIND, MU>, grid, 192, st, a, parity);
+  else su3c_split_kernel<FIELD, KIND, MU><<<grid, 192, 0, st>>>(a, parity);
+}
+
+template <int FIELD, int KIND, int MU>
 inline void su3c_launch_one(const Ctx& a, int parity, int block, cudaStream_t st) {
+  if (su3c_split(a.g)) return su3c_launch_split<FIELD, KIND, MU>(a, parity, st);
   launch_programmatic(su3c_phase_kernel<FIELD, KIND, MU>, grid_for(a.g.Vh, block), block, st, a, parity);
 }
 
@@ -571,15 +696,16 @@ inline void su3c_launch_level(const Ctx& a, int parity, int mu, int block, cudaS
   }
 }
 
-// The overrelaxation kernels that also reunitarize (last pass of a sweep),
-// with or without the fused plaquette sums, are compiled in their own
-// translation unit.
+// The heat-bath kernels and the overrelaxation kernels that also reunitarize
+// (last pass of a sweep), with or without the fused plaquette sums, are compiled
+// in translation units of their own.
+cudaError_t su3c_launch_hb(const Ctx& a, int parity, int mu, int block, cudaStream_t st);
 cudaError_t su3c_launch_or_reunit(const Ctx& a, int parity, int mu, int block, cudaStream_t st);
 cudaError_t su3c_launch_or_meas(const Ctx& a, int parity, int mu, int block, cudaStream_t st);
 
 inline cudaError_t su3c_launch_phase(const Ctx& a, int kind, int parity, int mu, int block, cudaStream_t st) {
-  if (kind == KIND_HB) su3c_launch_level<KIND_HB>(a, parity, mu, block, st);
-  else if (kind == KIND_OR) su3c_launch_level<KIND_OR>(a, parity, mu, block, st);
+  if (kind == KIND_HB) return su3c_launch_hb(a, parity, mu, block, st);
+  if (kind == KIND_OR) su3c_launch_level<KIND_OR>(a, parity, mu, block, st);
   else if (kind == KIND_OR_MEAS && mu >= 1) return su3c_launch_or_meas(a, parity, mu, block, st);
   else return su3c_launch_or_reunit(a, parity, mu, block, st);
   return cudaGetLastError();
@@ -598,13 +724,17 @@ int su3c_block_limit_mu() {
                   std::min(su3c_block_limit<FIELD, KIND, 2>(), su3c_block_limit<FIELD, KIND, 3>()));
 }
 
+int su3c_hb_max_block();
 int su3c_or_reunit_max_block();
 
+template <int KIND>
+int su3c_block_limit_level() {
+  return std::min(std::min(su3c_block_limit_mu<0, KIND>(), su3c_block_limit_mu<1, KIND>()),
+                  su3c_block_limit_mu<2, KIND>());
+}
+
 inline int su3c_max_phase_block() {
-  int m = std::min(std::min(su3c_block_limit_mu<0, KIND_HB>(), su3c_block_limit_mu<1, KIND_HB>()),
-                   std::min(su3c_block_limit_mu<0, KIND_OR>(), su3c_block_limit_mu<1, KIND_OR>()));
-  m = std::min(m, std::min(su3c_block_limit_mu<2, KIND_HB>(), su3c_block_limit_mu<2, KIND_OR>()));
-  return std::min(m, su3c_or_reunit_max_block());
+  return std::min(su3c_block_limit_level<KIND_OR>(), std::min(su3c_hb_max_block(), su3c_or_reunit_max_block()));
 }
 
 }  // namespace qcd

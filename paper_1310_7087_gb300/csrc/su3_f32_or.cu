@@ -11,6 +11,7 @@ cudaError_t su3c_launch_or_reunit(const Ctx& a, int parity, int mu, int block, c
 
 template <int FIELD, int MU>
 inline void launch_or_meas_one(const Ctx& a, int parity, int block, cudaStream_t st) {
+  if (su3c_split(a.g)) return su3c_launch_split<FIELD, KIND_OR_MEAS, MU>(a, parity, st);
   launch_programmatic(su3c_or_meas_kernel<FIELD, MU>, grid_for(a.g.Vh, block), block, st, a, parity);
 }
 
@@ -44,8 +45,7 @@ int or_meas_limit_mu() {
 }
 
 int su3c_or_reunit_max_block() {
-  int m = std::min(std::min(su3c_block_limit_mu<0, KIND_OR_REUNIT>(), su3c_block_limit_mu<1, KIND_OR_REUNIT>()),
-                   su3c_block_limit_mu<2, KIND_OR_REUNIT>());
+  const int m = su3c_block_limit_level<KIND_OR_REUNIT>();
   return std::min(m, std::min(std::min(or_meas_limit_mu<0>(), or_meas_limit_mu<1>()), or_meas_limit_mu<2>()));
 }
 }  // namespace qcd
