@@ -338,21 +338,21 @@ static __device__ __noinline__ float su3c_kp_retry(float inv_alpha, int nhit, St
 // beta > 0 and would otherwise sit in the hot code.
 static __device__ __noinline__ Quat<float> su3c_haar_rotation(Stream dir) { return su2_haar<float>(dir, 0u); }
 
-// Heat-bath or overrelaxation of U_MU(x) given its staple sum A.
+// Heat-bath or overrelaxation of U_mu(x) given its staple sum A.
 // Returns the link as stored (rows 0-1; row 2 not kept up to date).
-template <int FIELD, int KIND, int MU>
-__device__ __forceinline__ M3<float> su3c_update(const Ctx& a, int parity, int h, const LexSite& x,
+template <int FIELD, int KIND>
+__device__ __forceinline__ M3<float> su3c_update(const Ctx& a, int parity, int mu, int h, const LexSite& x,
                                                  const M3<float>& A, M3<float> U, const KpFirst* first = nullptr,
                                                  uint32_t sweep = 0) {
   M3<float> Ut = U;
-  if (FIELD == 2 && MU == 1) {
+  if (FIELD == 2 && mu == 1) {
     Cx<float> b[3];
     load_bdiag<float>(a, x.c[0], b);
 #pragma unroll
     for (int r = 0; r < 3; ++r)
 #pragma unroll
       for (int k = 0; k < 3; ++k) Ut.e[r][k] = cmul_pm(U.e[r][k], b[k]);
-  } else if (FIELD == 1 && MU == 1) {
+  } else if (FIELD == 1 && mu == 1) {
     const float2 ph = __ldg(a.phase32 + x.c[0]);
     const Cx<float> p{ph.x, ph.y}, pc{ph.x, -ph.y};
 #pragma unroll
@@ -374,11 +374,11 @@ __device__ __forceinline__ M3<float> su3c_update(const Ctx& a, int parity, int h
       const float rk = n2 > 0.f ? rsqrtf(n2) : 0.f;  // 1/k (approximate, ~2 ulp)
       const float k = n2 * rk;
       const float alpha = float(2.0 / 3.0) * float(a.beta) * k;
-      const Stream dir = make_stream(a.k0, a.k1, uint32_t(x.s), sweep, MU, sub, KIND_DIR);
+      const Stream dir = make_stream(a.k0, a.k1, uint32_t(x.s), sweep, mu, sub, KIND_DIR);
       if (alpha == 0.f) {
         r = su3c_haar_rotation(dir);
       } else {
-        const Stream tries = make_stream(a.k0, a.k1, uint32_t(x.s), sweep, MU, sub, KIND_TRY);
+        const Stream tries = make_stream(a.k0, a.k1, uint32_t(x.s), sweep, mu, sub, KIND_TRY);
         const float inv_alpha = __fdividef(1.f, alpha);
         float delta = first[sub].e * inv_alpha;
         if (!(first[sub].a3 <= 1.f - 0.5f * delta)) {
@@ -403,7 +403,7 @@ __device__ __forceinline__ M3<float> su3c_update(const Ctx& a, int parity, int h
   }
   if (exhausted) atomicAdd(a.exhausted, (unsigned long long)exhausted);
   if (KIND == KIND_OR_REUNIT || KIND == KIND_OR_MEAS) su3_reunit_value<float>(U);
-  SU3Policy<float>::store(a.links, a.g, MU, parity, h, U);
+  SU3Policy<float>::store(a.links, a.g, mu, parity, h, U);
   return U;
 }
 
@@ -447,8 +447,7 @@ __global__ void __maxnreg__(KIND == KIND_HB          ? QCD_SU3_HB_MAXNREG
                                  make_stream(a.k0, a.k1, uint32_t(x.s), sweep, MU, sub, KIND_DIR));
   }
   const M3<float> A = su3c_staple<FIELD, MU>(a, parity, x);
-  su3c_update<FIELD, KIND, MU>(a, parity, h, x, A, su3c_full(su3c_load(a.links, a.g, MU, parity, h)), first,
-                               sweep);
+  su3c_update<FIELD, KIND>(a, parity, MU, h, x, A, su3c_full(su3c_load(a.links, a.g, MU, parity, h)), first, sweep);
 }
 
 // Last-pass phase (odd parity, MU >= 1) of a working sweep: update and
@@ -463,10 +462,11 @@ __global__ void __maxnreg__(KIND == KIND_HB          ? QCD_SU3_HB_MAXNREG
 #endif
 
 // Re Tr(Ut low) of an updated link (the final sums take the 1/3).
-template <int FIELD, int MU>
-__device__ __forceinline__ float su3c_plane_sum(const Ctx& a, const LexSite& x, M3<float> U, const M3<float>& low) {
+template <int FIELD>
+__device__ __forceinline__ float su3c_plane_sum(const Ctx& a, int mu, const LexSite& x, M3<float> U,
+                                                const M3<float>& low) {
   su3c_rebuild(U);  // row 2 as every later load rebuilds it
-  if (FIELD == 1 && MU == 1) {
+  if (FIELD == 1 && mu == 1) {
     const float2 ph = __ldg(a.phase32 + x.c[0]);
     const Cx<float> pp{ph.x, ph.y}, pc{ph.x, -ph.y};
 #pragma unroll
@@ -474,7 +474,7 @@ __device__ __forceinline__ float su3c_plane_sum(const Ctx& a, const LexSite& x, 
       U.e[r][0] = cmul_pm(U.e[r][0], pp);
       U.e[r][1] = cmul_pm(U.e[r][1], pc);
     }
-  } else if (FIELD == 2 && MU == 1) {
+  } else if (FIELD == 2 && mu == 1) {
     Cx<float> b[3];
     load_bdiag<float>(a, x.c[0], b);
 #pragma unroll
@@ -496,9 +496,9 @@ __global__ void __maxnreg__(QCD_SU3_MEAS_MAXNREG) su3c_or_meas_kernel(const Ctx 
     const int h = x.s >> 1;
     M3<float> low;
     const M3<float> A = su3c_staple<FIELD, MU, true>(a, parity, x, &low);
-    M3<float> U = su3c_update<FIELD, KIND_OR_MEAS, MU>(a, parity, h, x, A,
-                                                       su3c_full(su3c_load(a.links, a.g, MU, parity, h)));
-    v = su3c_plane_sum<FIELD, MU>(a, x, U, low);
+    M3<float> U = su3c_update<FIELD, KIND_OR_MEAS>(a, parity, MU, h, x, A,
+                                                   su3c_full(su3c_load(a.links, a.g, MU, parity, h)));
+    v = su3c_plane_sum<FIELD>(a, MU, x, U, low);
   }
   block_sum_f32(v, a.partials + fused_plaq_offset(a.g, MU) + blockIdx.x);
 }
@@ -506,44 +506,75 @@ __global__ void __maxnreg__(QCD_SU3_MEAS_MAXNREG) su3c_or_meas_kernel(const Ctx 
 // Small lattices: six warps share 32 links (lane = link), each computes one staple;
 // warp 0 adds them up in the order of su3c_staple, so that the results are the
 // same to the bit, and updates the links.  The heat-bath's draws ahead are spread
-// over warps 3 to 5.
+// over warps 3 to 5.  The directions are run-time values: one kernel serves the
+// four phases of a parity and its two staple bodies the six warps, so the code
+// stays in the instruction caches from phase to phase (a kernel per direction with
+// a body per staple took 144 / 159 / 232 us per sweep at 12^3x4 / 16^3x4 / 20^3x4,
+// this one 127 / 138 / 222).
 struct Su3cSplitShared {
   float4 t[6][3][32];
   float first[3][6][32];
 };
 
-template <int FIELD, int KIND, int MU>
-__global__ void __launch_bounds__(192, 3) su3c_split_kernel(const Ctx a, int parity) {
+template <int FIELD>
+__device__ __forceinline__ Rows2 su3c_eff_at(const Ctx& a, int d, int par, int s, int x) {
+  Rows2 r = su3c_load(a.links, a.g, d, par, s >> 1);
+  if (FIELD == 1 && d == 1) {
+    const float2 ph = __ldg(a.phase32 + x);
+    su3c_phase(r, ph.x, ph.y);
+  } else if (FIELD == 2 && d == 1) {
+    Cx<float> b[3];
+    load_bdiag<float>(a, x, b);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) r.e[i][k] = cmul_pm(r.e[i][k], b[k]);
+  }
+  return r;
+}
+
+template <int FIELD, int KIND>
+__global__ void __launch_bounds__(192, 3) su3c_split_kernel(const Ctx a, int parity, int mu) {
   pdl_launch_dependents();
   __shared__ Su3cSplitShared sh;
   const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + lane;
   const bool in = i < a.g.Vh;
   const LexSite x = lex_site_ytz(a.g, parity, in ? i : a.g.Vh - 1);
-  const bool on = in && !frozen_link(a, MU, x.c[3]);
-  const LexSite xp = lex_step<MU, +1>(a.g, x);
+  const bool on = in && !frozen_link(a, mu, x.c[3]);
+  const int n = role >> 1, nu = n + (n >= mu);
+  const bool lower = role & 1;
+  // one step of site s along d; only x-steps change the coordinate that the
+  // background needs
+  auto stride = [&](int d) { return d == 0 ? 1 : d == 1 ? a.g.Ns : d == 2 ? a.g.Ns * a.g.Ns : a.g.Ns * a.g.Ns * a.g.Ns; };
+  auto coord = [&](int d) { return d == 0 ? x.c[0] : d == 1 ? x.c[1] : d == 2 ? x.c[2] : x.c[3]; };
+  const int st_mu = stride(mu), st_nu = stride(nu), c_mu = coord(mu), c_nu = coord(nu);
+  const int e_mu = mu == 3 ? a.g.Nt : a.g.Ns, e_nu = nu == 3 ? a.g.Nt : a.g.Ns;
+  const int up = c_mu == e_mu - 1 ? st_mu - e_mu * st_mu : st_mu;
+  const int off = lower ? (c_nu == 0 ? e_nu * st_nu - st_nu : -st_nu) : (c_nu == e_nu - 1 ? st_nu - e_nu * st_nu : st_nu);
+  const int x_mu = x.c[0] + (mu == 0 ? up : 0), x_nu = x.c[0] + (nu == 0 ? off : 0);
   pdl_wait();
   uint32_t sweep = 0;
   if (KIND == KIND_HB) sweep = *a.sweep;
   Rows2 own;
-  if (role == 0) own = su3c_load(a.links, a.g, MU, parity, x.s >> 1);
+  if (role == 0) own = su3c_load(a.links, a.g, mu, parity, x.s >> 1);
   Rows2 t;
-  switch (role) {
-#define QCD_SU3C_ROLE(N)                                                                                  \
-  case 2 * N: t = su3c_one_staple<FIELD, MU, N + (N >= MU), false>(a, parity, x, xp); break;               \
-  case 2 * N + 1: t = su3c_one_staple<FIELD, MU, N + (N >= MU), true>(a, parity, x, xp); break;
-    QCD_SU3C_ROLE(0)
-    QCD_SU3C_ROLE(1)
-    QCD_SU3C_ROLE(2)
-#undef QCD_SU3C_ROLE
+  if (!lower) {
+    const Rows2 x1 = su3c_mul_nd(su3c_eff_at<FIELD>(a, nu, parity ^ 1, x.s + up, x_mu),
+                                 su3c_full(su3c_eff_at<FIELD>(a, mu, parity ^ 1, x.s + off, x_nu)));
+    t = su3c_mul_nd(x1, su3c_full(su3c_eff_at<FIELD>(a, nu, parity, x.s, x.c[0])));
+  } else {
+    const M3<float> y = su3c_full(su3c_mul(su3c_eff_at<FIELD>(a, mu, parity ^ 1, x.s + off, x_nu),
+                                           su3c_full(su3c_eff_at<FIELD>(a, nu, parity, x.s + up + off, x_mu))));
+    t = su3c_mul_dn(y, su3c_full(su3c_eff_at<FIELD>(a, nu, parity ^ 1, x.s + off, x.c[0])));
   }
   sh.t[role][0][lane] = make_float4(t.e[0][0].re, t.e[0][0].im, t.e[0][1].re, t.e[0][1].im);
   sh.t[role][1][lane] = make_float4(t.e[0][2].re, t.e[0][2].im, t.e[1][0].re, t.e[1][0].im);
   sh.t[role][2][lane] = make_float4(t.e[1][1].re, t.e[1][1].im, t.e[1][2].re, t.e[1][2].im);
   if (KIND == KIND_HB && role >= 3) {
     const int sub = role - 3;
-    const KpFirst f = su3c_kp_first(make_stream(a.k0, a.k1, uint32_t(x.s), sweep, MU, sub, KIND_TRY),
-                                    make_stream(a.k0, a.k1, uint32_t(x.s), sweep, MU, sub, KIND_DIR));
+    const KpFirst f = su3c_kp_first(make_stream(a.k0, a.k1, uint32_t(x.s), sweep, mu, sub, KIND_TRY),
+                                    make_stream(a.k0, a.k1, uint32_t(x.s), sweep, mu, sub, KIND_DIR));
     sh.first[sub][0][lane] = f.e;
     sh.first[sub][1][lane] = f.a3;
     sh.first[sub][2][lane] = f.st;
@@ -555,12 +586,9 @@ __global__ void __launch_bounds__(192, 3) su3c_split_kernel(const Ctx a, int par
   if (role > 0) return;
   M3<float> A, low;
   m3_zero(A);
-#pragma unroll
+  low = A;
+#pragma unroll 1
   for (int s = 0; s < 6; ++s) {
-    if (KIND == KIND_OR_MEAS && s == 2 * MU) {
-      low = A;
-      su3c_conj_row2(low);
-    }
     const float4 u = sh.t[s][0][lane], v = sh.t[s][1][lane], w = sh.t[s][2][lane];
     Rows2 r;
     r.e[0][0] = {u.x, u.y};
@@ -570,11 +598,9 @@ __global__ void __launch_bounds__(192, 3) su3c_split_kernel(const Ctx a, int par
     r.e[1][1] = {w.x, w.y};
     r.e[1][2] = {w.z, w.w};
     su3c_acc_c(A, r);
+    if (KIND == KIND_OR_MEAS && s == 2 * mu - 1) low = A;
   }
-  if (KIND == KIND_OR_MEAS && MU == 3) {
-    low = A;
-    su3c_conj_row2(low);
-  }
+  if (KIND == KIND_OR_MEAS) su3c_conj_row2(low);
   su3c_conj_row2(A);
   KpFirst first[3];
   if (KIND == KIND_HB)
@@ -584,19 +610,19 @@ __global__ void __launch_bounds__(192, 3) su3c_split_kernel(const Ctx a, int par
                     sh.first[sub][3][lane], sh.first[sub][4][lane], sh.first[sub][5][lane]};
   SumF v;
   if (on) {
-    M3<float> U = su3c_update<FIELD, KIND, MU>(a, parity, x.s >> 1, x, A, su3c_full(own), first, sweep);
-    if (KIND == KIND_OR_MEAS) v.s = su3c_plane_sum<FIELD, MU>(a, x, U, low);
+    const M3<float> U = su3c_update<FIELD, KIND>(a, parity, mu, x.s >> 1, x, A, su3c_full(own), first, sweep);
+    if (KIND == KIND_OR_MEAS) v.s = su3c_plane_sum<FIELD>(a, mu, x, U, low);
   }
   if (KIND == KIND_OR_MEAS) {
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v.merge_down(off);
-    if (lane == 0) a.partials[fused_plaq_offset(a.g, MU) + blockIdx.x] = v.value();
+    for (int off2 = 16; off2 > 0; off2 >>= 1) v.merge_down(off2);
+    if (lane == 0) a.partials[fused_plaq_offset(a.g, mu) + blockIdx.x] = v.value();
   }
 }
 
 // Split up to 800 CTAs of 32 links: sweeps of 1 heat-bath + 4 overrelaxation
-// passes, us, not split / split: 4^3x4 229 / 115, 12^3x4 (108 CTAs) 230 / 144, 16^3x4
-// (256) 240 / 159, 20^3x4 (500) 289 / 232, 20^3x6 (750) 288 / 255, 24^3x6 (1296) 326 /
+// passes, us, not split / split: 4^3x4 229 / 113, 12^3x4 (108 CTAs) 230 / 127, 16^3x4
+// (256) 240 / 138, 20^3x4 (500) 289 / 222, 20^3x6 (750) 288 / 258, 24^3x6 (1296) 326 /
 // 349.  At these sizes a phase is one chain of latencies (one warp per SM
 // sub-partition or less): the gather's loads, 12 products one after another, the
 // update; the split takes the products and most of the loads out of the chain.
@@ -645,9 +671,8 @@ inline cudaError_t su3c_measure_fused_tail(const Ctx& a, int block, cudaStream_t
 // Launch with programmatic stream serialization: the kernel may be scheduled
 // before its predecessor in the stream (or in the captured graph) completes;
 // it waits in-kernel (pdl_wait) before touching the predecessor's results.
-template <typename... P>
-inline void launch_programmatic(void (*kernel)(P...), unsigned grid, int block, cudaStream_t st, const Ctx& a,
-                                int parity) {
+template <typename... P, typename... A>
+inline void launch_programmatic(void (*kernel)(P...), unsigned grid, int block, cudaStream_t st, A... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(unsigned(block));
@@ -658,27 +683,27 @@ inline void launch_programmatic(void (*kernel)(P...), unsigned grid, int block, 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, kernel, a, parity);
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
-template <int FIELD, int KIND, int MU>
-inline void su3c_launch_split(const Ctx& a, int parity, cudaStream_t st) {
+template <int FIELD, int KIND>
+inline void su3c_launch_split(const Ctx& a, int parity, int mu, cudaStream_t st) {
   // Programmatic launch beyond one wave of 3 CTAs per SM (20^3x4: 246 -> 232 us per
   // sweep); within one it places the next phase's CTAs on the SMs that are left
   // (4^3x4: 115 -> 136).
   const unsigned grid = grid_for(a.g.Vh, 32);
-  if (grid > 3 * 152) launch_programmatic(su3c_split_kernel<FIELD, KIND, MU>, grid, 192, st, a, parity);
-  else su3c_split_kernel<FIELD, KIND, MU><<<grid, 192, 0, st>>>(a, parity);
+  if (grid > 3 * 152) launch_programmatic(su3c_split_kernel<FIELD, KIND>, grid, 192, st, a, parity, mu);
+  else su3c_split_kernel<FIELD, KIND><<<grid, 192, 0, st>>>(a, parity, mu);
 }
 
 template <int FIELD, int KIND, int MU>
 inline void su3c_launch_one(const Ctx& a, int parity, int block, cudaStream_t st) {
-  if (su3c_split(a.g)) return su3c_launch_split<FIELD, KIND, MU>(a, parity, st);
   launch_programmatic(su3c_phase_kernel<FIELD, KIND, MU>, grid_for(a.g.Vh, block), block, st, a, parity);
 }
 
 template <int FIELD, int KIND>
 inline void su3c_launch_kind(const Ctx& a, int parity, int mu, int block, cudaStream_t st) {
+  if (su3c_split(a.g)) return su3c_launch_split<FIELD, KIND>(a, parity, mu, st);
   switch (mu) {
     case 0: su3c_launch_one<FIELD, KIND, 0>(a, parity, block, st); break;
     case 1: su3c_launch_one<FIELD, KIND, 1>(a, parity, block, st); break;

@@ -11,12 +11,12 @@ cudaError_t su3c_launch_or_reunit(const Ctx& a, int parity, int mu, int block, c
 
 template <int FIELD, int MU>
 inline void launch_or_meas_one(const Ctx& a, int parity, int block, cudaStream_t st) {
-  if (su3c_split(a.g)) return su3c_launch_split<FIELD, KIND_OR_MEAS, MU>(a, parity, st);
   launch_programmatic(su3c_or_meas_kernel<FIELD, MU>, grid_for(a.g.Vh, block), block, st, a, parity);
 }
 
 template <int FIELD>
 inline void launch_or_meas_mu(const Ctx& a, int parity, int mu, int block, cudaStream_t st) {
+  if (su3c_split(a.g)) return su3c_launch_split<FIELD, KIND_OR_MEAS>(a, parity, mu, st);
   switch (mu) {
     case 1: launch_or_meas_one<FIELD, 1>(a, parity, block, st); break;
     case 2: launch_or_meas_one<FIELD, 2>(a, parity, block, st); break;
