@@ -77,28 +77,33 @@ __device__ __forceinline__ void su2d_staple(const Ctx& a, int p, const LexSite& 
 }
 
 // The update in FP64, out of line: links outside the fixed-point range.
-template <bool FIELD, int KIND, int MU, bool CG>
-__device__ __noinline__ double su2d_general(Ctx a, int parity, LexSite x, uint32_t sweep) {
-  return su2c_update_at<double, FIELD, KIND, MU, CG>(a, parity, x, sweep);
+template <bool FIELD, int KIND, bool CG>
+__device__ __noinline__ double su2d_general(Ctx a, int parity, int mu, LexSite x, uint32_t sweep) {
+  switch (mu) {
+    case 0: return su2c_update_at<double, FIELD, KIND, 0, CG>(a, parity, x, sweep);
+    case 1: return su2c_update_at<double, FIELD, KIND, 1, CG>(a, parity, x, sweep);
+    case 2: return su2c_update_at<double, FIELD, KIND, 2, CG>(a, parity, x, sweep);
+    default: return su2c_update_at<double, FIELD, KIND, 3, CG>(a, parity, x, sweep);
+  }
 }
 
 static __device__ __noinline__ Quat<double> su2d_haar(Stream dir) { return su2_haar<double>(dir, 0u); }
 
 // One link update given its staple sum A (and the part of it over nu < MU), as
 // su2c_update_at.
-template <bool FIELD, int KIND, int MU, bool CG>
-__device__ __forceinline__ double su2d_update(const Ctx& a, int parity, const LexSite& x, uint32_t sweep,
+template <bool FIELD, int KIND, bool CG>
+__device__ __forceinline__ double su2d_update(const Ctx& a, int parity, int mu, const LexSite& x, uint32_t sweep,
                                               int64_t A[4], const int64_t low[4], uint32_t big, uint32_t bad,
                                               const FxKpFirst* first) {
   constexpr bool reunit = KIND == KIND_OR_REUNIT || KIND == KIND_OR_MEAS;
   constexpr bool meas = KIND == KIND_OR_MEAS;
-  constexpr bool phased = FIELD && MU == 1;
+  const bool phased = FIELD && mu == 1;
   using P = SU2Policy<double>;
   Fx u[4];
   bool keep = false;
   if (KIND == KIND_HB) {
-    if ((bad & FX_BAD) || (big & FX_BIG)) return su2d_general<FIELD, KIND, MU, CG>(a, parity, x, sweep);
-    const Stream dir = make_stream(a.k0, a.k1, uint32_t(x.s), sweep, MU, 0, KIND_DIR);
+    if ((bad & FX_BAD) || (big & FX_BIG)) return su2d_general<FIELD, KIND, CG>(a, parity, mu, x, sweep);
+    const Stream dir = make_stream(a.k0, a.k1, uint32_t(x.s), sweep, mu, 0, KIND_DIR);
     if (a.beta == 0.0 || (A[0] | A[1] | A[2] | A[3]) == 0) {
       const Quat<double> R = su2d_haar(dir);
       u[0] = fx_load(R.q0, big);
@@ -106,16 +111,16 @@ __device__ __forceinline__ double su2d_update(const Ctx& a, int parity, const Le
       u[2] = fx_load(R.q2, big);
       u[3] = fx_load(R.q3, big);
     } else {
-      const Stream tries = make_stream(a.k0, a.k1, uint32_t(x.s), sweep, MU, 0, KIND_TRY);
+      const Stream tries = make_stream(a.k0, a.k1, uint32_t(x.s), sweep, mu, 0, KIND_TRY);
       if (!fx_heatbath(A, 1.0 / a.beta, a.nhit, tries, *first, u)) {
         atomicAdd(a.exhausted, 1ull);
         return 0.0;  // the link stays as it is
       }
     }
   } else {
-    su2d_load<false, CG>(a, MU, parity, x.s, u, big);
+    su2d_load<false, CG>(a, mu, parity, x.s, u, big);
     if (phased) su2d_phase<false, false>(a, x.c[0], u, bad);
-    if ((bad & FX_BAD) || (big & FX_BIG)) return su2d_general<FIELD, KIND, MU, CG>(a, parity, x, sweep);
+    if ((bad & FX_BAD) || (big & FX_BIG)) return su2d_general<FIELD, KIND, CG>(a, parity, mu, x, sweep);
     // V^+ U^+ V^+ = 2 <V^+, U> V^+ - U for the unit quaternion V = A / |A|
     if (fx_normalise4(A)) {
       Fx w[4];
@@ -136,7 +141,7 @@ __device__ __forceinline__ double su2d_update(const Ctx& a, int parity, const Le
         t.add(w[k], s);
         u[k] = fx_limbs(fx_sub(2 * t.value(), fx_value(u[k])));
       }
-      if (bad & FX_BAD) return su2d_general<FIELD, KIND, MU, CG>(a, parity, x, sweep);
+      if (bad & FX_BAD) return su2d_general<FIELD, KIND, CG>(a, parity, mu, x, sweep);
     } else {
       keep = true;
     }
@@ -163,7 +168,7 @@ __device__ __forceinline__ double su2d_update(const Ctx& a, int parity, const Le
     u[2] = fx_load(q.q2, big);
     u[3] = fx_load(q.q3, big);
   }
-  P::store(a.links, a.g, MU, parity, x.s >> 1, q);
+  P::store(a.links, a.g, mu, parity, x.s >> 1, q);
   if (!meas) return 0.0;
   if (phased) su2d_phase<false, false>(a, x.c[0], u, bad);
   FxAcc t;  // (1/2) Re Tr(Ut low) / 8
@@ -205,115 +210,145 @@ __device__ __forceinline__ double su2d_update_at(const Ctx& a, int parity, const
   if (KIND == KIND_HB)
     first = fx_kp_first(make_stream(a.k0, a.k1, uint32_t(x.s), sweep, MU, 0, KIND_TRY),
                         make_stream(a.k0, a.k1, uint32_t(x.s), sweep, MU, 0, KIND_DIR));
-  return su2d_update<FIELD, KIND, MU, CG>(a, parity, x, sweep, A, low, big, bad, &first);
-}
-
-// One staple, chosen by s (uniform in a warp).
-template <bool FIELD, int MU, bool CG>
-__device__ __forceinline__ void su2d_one_staple(const Ctx& a, int p, const LexSite& x, int s, int64_t A[4],
-                                                uint32_t& big, uint32_t& bad) {
-  switch (s) {
-#define QCD_SU2D_ONE(N)                                                                                          \
-  case 2 * N: su2d_staple<FIELD, MU, N + (N >= MU), false, CG>(a, p, x, A, big, bad); break;              \
-  case 2 * N + 1: su2d_staple<FIELD, MU, N + (N >= MU), true, CG>(a, p, x, A, big, bad); break;
-    QCD_SU2D_ONE(0)
-    QCD_SU2D_ONE(1)
-    QCD_SU2D_ONE(2)
-#undef QCD_SU2D_ONE
-  }
+  return su2d_update<FIELD, KIND, CG>(a, parity, MU, x, sweep, A, low, big, bad, &first);
 }
 
 // Bound: integer pipe and FP64 unit together (ncu at 32^3x8, overrelaxation of
 // t-links: ALU 45 %, 3,390 instructions per update) where the FP64 form was bound
 // by the FP64 unit.  Phase times, us, FP64 form -> this, overrelaxation /
-// heat-bath of y-links: 4^3x4 14.4 / 30.8 -> 6.4 / 10.6; 32^3x8 77 / 159 -> 31 / 45;
+// heat-bath of y-links: 32^3x8 77 / 159 -> 31 / 45;
 // 64^3x16 1104 / 2135 -> 440 / 661.  128 registers: 96 / 80 / 64 gave sweeps of
 // 8.2 / 8.5 / 9.4 ms at 64^3x16 against 8.2, and 572 / 640 / 613 us at 32^3x8
 // against 534.
 //
-// SPLIT = 1: one thread per link.  SPLIT = 6: six warps share 32 links, each
-// taking one staple; the integer sums are exact, so the results are the same.
-template <bool FIELD, int KIND, int MU, int SPLIT>
+// One thread per link.
+template <bool FIELD, int KIND, int MU>
 __global__ void __maxnreg__(128) su2d_phase_kernel(const __grid_constant__ Ctx a, int parity) {
-  double v = 0.0;
-  if (SPLIT == 1) {
-    const int h = blockIdx.x * blockDim.x + threadIdx.x;
-    if (h < a.g.Vh)
-      v = su2d_update_at<FIELD, KIND, MU, false>(a, parity, lex_site(a, parity, h), KIND == KIND_HB ? *a.sweep : 0u);
-  } else {
-    __shared__ int64_t part[SPLIT][4][32];
-    __shared__ uint32_t flag[SPLIT][32];
-    const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
-    const int h = blockIdx.x * 32 + lane;
-    const bool in = h < a.g.Vh;
-    const LexSite x = lex_site(a, parity, in ? h : a.g.Vh - 1);
-    const bool on = in && !frozen_link(a, MU, x.c[3]);
-    const uint32_t sweep = KIND == KIND_HB ? *a.sweep : 0u;
-    int64_t A[4] = {};
-    uint32_t big = 0, bad = 0;
-    FxKpFirst first;
-    su2d_one_staple<FIELD, MU, false>(a, parity, x, role, A, big, bad);
-    if (role > 0) {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) part[role][k][lane] = A[k];
-      flag[role][lane] = (bad & FX_BAD) | (big & FX_BIG);
-    } else if (KIND == KIND_HB) {
-      first = fx_kp_first(make_stream(a.k0, a.k1, uint32_t(x.s), sweep, MU, 0, KIND_TRY),
-                          make_stream(a.k0, a.k1, uint32_t(x.s), sweep, MU, 0, KIND_DIR));
-    }
-    __syncthreads();
-    if (role > 0) return;
-    int64_t low[4] = {};
-#pragma unroll
-    for (int s = 0; s < 6; ++s) {
-      if (s > 0) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) A[k] += part[s][k][lane];
-        bad |= flag[s][lane] & FX_BAD;
-        big |= flag[s][lane] & FX_BIG;
-      }
-      if (KIND == KIND_OR_MEAS && s == 2 * MU - 1)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) low[k] = A[k];
-    }
-    if (on) v = su2d_update<FIELD, KIND, MU, false>(a, parity, x, sweep, A, low, big, bad, &first);
-  }
-  if (KIND == KIND_OR_MEAS) {
-    double* out = a.partials + fused_plaq_offset(a.g, MU) + blockIdx.x;
-    if (SPLIT == 1) {
-      SumD s[1];
-      s[0].s = v;
-      block_sums(s, out);
-    } else {  // one warp is left
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-      if (threadIdx.x == 0) *out = v;
-    }
-  }
+  SumD v[1];
+  const int h = blockIdx.x * blockDim.x + threadIdx.x;
+  if (h < a.g.Vh)
+    v[0].s = su2d_update_at<FIELD, KIND, MU, false>(a, parity, lex_site(a, parity, h), KIND == KIND_HB ? *a.sweep : 0u);
+  if (KIND == KIND_OR_MEAS) block_sums(v, a.partials + fused_plaq_offset(a.g, MU) + blockIdx.x);
 }
 
-// Split up to one CTA of 32 links per SM (152): sweeps of 1 heat-bath + 1
-// overrelaxation pass, us, split / not: 4^3x4 91 / 145, 8^3x4 105 / 150, 12^3x4
-// (108 CTAs) 137 / 150, 20^3x4 (500) 242 / 160.
-inline bool su2d_split(const GeomH& g) { return (g.Vh + 31) / 32 <= 152; }
-// Links of one CTA for a block size of the caller.
-inline int su2d_links_per_cta(const GeomH& g, int block) { return su2d_split(g) ? 32 : block; }
-
-template <bool FIELD, int KIND, int MU>
-inline void su2d_launch_one(const Ctx& a, int parity, int block, cudaStream_t st) {
-  if (su2d_split(a.g)) su2d_phase_kernel<FIELD, KIND, MU, 6><<<grid_for(a.g.Vh, 32), 192, 0, st>>>(a, parity);
-  else su2d_phase_kernel<FIELD, KIND, MU, 1><<<grid_for(a.g.Vh, block), block, 0, st>>>(a, parity);
+// Small lattices: six warps share 32 links, each taking one staple; the integer
+// sums are exact, so the results are the same.  The directions are run-time values
+// and the two kinds of staple one body (the adjoint of a link by the sign of its
+// imaginary quaternion parts), so that the code stays in the instruction caches
+// from phase to phase (a kernel per direction with a body per staple took 91 / 137 /
+// 160 us per sweep at 4^3x4 / 12^3x4 / 16^3x4, this one 84 / 95 / 104).
+__device__ __forceinline__ void su2d_load_at(const Ctx& a, int d, int par, int s, uint32_t dag, Fx q[4], uint32_t& big) {
+  const Quat<double> u = SU2Policy<double>::load(a.links, a.g, d, par, s >> 1);
+  const double v[4] = {u.q0, u.q1, u.q2, u.q3};
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    q[k] = fx_load_int(k ? __hiloint2double(__double2hiint(v[k]) ^ int(dag), __double2loint(v[k])) : v[k], big);
 }
 
 template <bool FIELD, int KIND>
+__global__ void __launch_bounds__(192) su2d_split_kernel(const __grid_constant__ Ctx a, int parity, int mu) {
+  __shared__ int64_t part[6][4][32];
+  __shared__ uint32_t flag[6][32];
+  __shared__ FxKpFirst ahead[32];
+  const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
+  const int h = blockIdx.x * 32 + lane;
+  const bool in = h < a.g.Vh;
+  const LexSite x = lex_site(a, parity, in ? h : a.g.Vh - 1);
+  const bool on = in && !frozen_link(a, mu, x.c[3]);
+  const uint32_t sweep = KIND == KIND_HB ? *a.sweep : 0u;
+  int64_t A[4] = {};
+  uint32_t big = 0, bad = 0;
+  {
+    const int n = role >> 1, nu = n + (n >= mu);
+    const bool lower = role & 1;
+    auto stride = [&](int d) { return d == 0 ? 1 : d == 1 ? a.g.Ns : d == 2 ? a.g.Ns * a.g.Ns : a.g.Ns * a.g.Ns * a.g.Ns; };
+    auto coord = [&](int d) { return d == 0 ? x.c[0] : d == 1 ? x.c[1] : d == 2 ? x.c[2] : x.c[3]; };
+    const int st_mu = stride(mu), st_nu = stride(nu), c_mu = coord(mu), c_nu = coord(nu);
+    const int e_mu = mu == 3 ? a.g.Nt : a.g.Ns, e_nu = nu == 3 ? a.g.Nt : a.g.Ns;
+    const int up = c_mu == e_mu - 1 ? st_mu - e_mu * st_mu : st_mu;
+    const int off =
+        lower ? (c_nu == 0 ? e_nu * st_nu - st_nu : -st_nu) : (c_nu == e_nu - 1 ? st_nu - e_nu * st_nu : st_nu);
+    const int base = lower ? x.s + off : x.s, pb = lower ? parity ^ 1 : parity;
+    const uint32_t sign = 0x80000000u;
+    // Ut_nu(x+mu) Ut_mu(x+nu)^+ Ut_nu(x)^+, Ut_nu(x+mu-nu)^+ Ut_mu(x-nu)^+ Ut_nu(x-nu)
+    Fx u[4], v[4], w[4];
+    su2d_load_at(a, nu, pb ^ 1, base + up, lower ? sign : 0u, u, big);
+    su2d_load_at(a, mu, parity ^ 1, x.s + off, sign, v, big);
+    su2d_load_at(a, nu, pb, base, lower ? 0u : sign, w, big);
+    if (FIELD && nu == 1) {
+      const int x_mu = x.c[0] + (mu == 0 ? up : 0);
+      if (lower) {
+        su2d_phase<true, false>(a, x_mu, u, bad);
+        su2d_phase<false, false>(a, x.c[0], w, bad);
+      } else {
+        su2d_phase<false, false>(a, x_mu, u, bad);
+        su2d_phase<true, false>(a, x.c[0], w, bad);
+      }
+    }
+    if (FIELD && mu == 1) su2d_phase<true, false>(a, x.c[0] + (nu == 0 ? off : 0), v, bad);
+    int64_t t[4];
+    fx_qmul(u, v, t);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      fx_check(t[k], bad);
+      u[k] = fx_limbs(t[k]);
+    }
+    fx_qmul(u, w, A);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) fx_check(A[k], bad);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) part[role][k][lane] = A[k];
+  flag[role][lane] = (bad & FX_BAD) | (big & FX_BIG);
+  if (KIND == KIND_HB && role == 5)
+    ahead[lane] = fx_kp_first(make_stream(a.k0, a.k1, uint32_t(x.s), sweep, mu, 0, KIND_TRY),
+                              make_stream(a.k0, a.k1, uint32_t(x.s), sweep, mu, 0, KIND_DIR));
+  __syncthreads();
+  if (role > 0) return;
+  int64_t low[4] = {};
+#pragma unroll
+  for (int s = 1; s < 6; ++s) {
+    if (KIND == KIND_OR_MEAS && s == 2 * mu)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) low[k] = A[k];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) A[k] += part[s][k][lane];
+    bad |= flag[s][lane] & FX_BAD;
+    big |= flag[s][lane] & FX_BIG;
+  }
+  if (KIND == KIND_OR_MEAS && mu == 3)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) low[k] = A[k];
+  double v = 0.0;
+  if (on) v = su2d_update<FIELD, KIND, false>(a, parity, mu, x, sweep, A, low, big, bad, &ahead[lane]);
+  if (KIND == KIND_OR_MEAS) {  // one warp is left
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (threadIdx.x == 0) a.partials[fused_plaq_offset(a.g, mu) + blockIdx.x] = v;
+  }
+}
+
+// Split up to 512 CTAs of 32 links: sweeps of 1 heat-bath + 1 overrelaxation pass,
+// us, split / not: 4^3x4 84 / 148, 12^3x4 (108 CTAs) 95 / 155, 16^3x4 (256) 104 / 158,
+// 20^3x4 (500) 156 / 162.
+inline bool su2d_split(const GeomH& g) { return (g.Vh + 31) / 32 <= 512; }
+// Links of one CTA for a block size of the caller.
+inline int su2d_links_per_cta(const GeomH& g, int block) { return su2d_split(g) ? 32 : block; }
+
+template <bool FIELD, int KIND>
 inline void su2d_launch_kind(const Ctx& a, int parity, int mu, int block, cudaStream_t st) {
+  const unsigned grid = grid_for(a.g.Vh, su2d_links_per_cta(a.g, block));
+  if (su2d_split(a.g)) {
+    su2d_split_kernel<FIELD, KIND><<<grid, 192, 0, st>>>(a, parity, mu);
+    return;
+  }
   switch (mu) {
     case 0:
-      if (KIND != KIND_OR_MEAS) su2d_launch_one<FIELD, KIND == KIND_OR_MEAS ? KIND_OR : KIND, 0>(a, parity, block, st);
+      if constexpr (KIND != KIND_OR_MEAS) su2d_phase_kernel<FIELD, KIND, 0><<<grid, block, 0, st>>>(a, parity);
       break;
-    case 1: su2d_launch_one<FIELD, KIND, 1>(a, parity, block, st); break;
-    case 2: su2d_launch_one<FIELD, KIND, 2>(a, parity, block, st); break;
-    default: su2d_launch_one<FIELD, KIND, 3>(a, parity, block, st); break;
+    case 1: su2d_phase_kernel<FIELD, KIND, 1><<<grid, block, 0, st>>>(a, parity); break;
+    case 2: su2d_phase_kernel<FIELD, KIND, 2><<<grid, block, 0, st>>>(a, parity); break;
+    default: su2d_phase_kernel<FIELD, KIND, 3><<<grid, block, 0, st>>>(a, parity); break;
   }
 }
 

@@ -37,7 +37,7 @@ def links_of(kind, links, rng):
 
 @pytest.mark.parametrize("kind", ["unitary", "scaled", "zero"])
 @pytest.mark.parametrize("group,Ns,Nt,flux,flux8", [(3, 6, 2, 1, 0), (3, 6, 6, 0, 0), (3, 18, 4, 1, 1), (3, 20, 4, 2, 0),
-                                                    (2, 6, 2, 1, 0), (2, 6, 6, 0, 0), (2, 18, 4, 2, 0)])
+                                                    (2, 6, 2, 1, 0), (2, 6, 6, 0, 0), (2, 18, 4, 2, 0), (2, 20, 6, 1, 0)])
 def test_phases(q, group, Ns, Nt, flux, flux8, kind):
     beta = 5.7 if group == 3 else 2.3
     lat = q.Lattice(group, Ns, Nt, beta, flux, FP64_PLAIN, HOT, 7, flux8=flux8)
