@@ -246,17 +246,22 @@ def qcd_measure_bare(h):
 
 
 def qcd_get_links(h, V: int, N: int) -> np.ndarray:
-    out = np.empty((V, 4, N, N, 2), np.float64)
-    _check(lib().qcd_get_links(h, _dptr(out)))
-    return out[..., 0] + 1j * out[..., 1]
+    out = np.empty((V, 4, N, N), np.complex128)
+    _check(lib().qcd_get_links(h, _dptr(out.view(np.float64))))
+    return out
+
+
+def _links_f64(links) -> np.ndarray:
+    """Contiguous FP64 reals of an array of complex links (no copy when it is
+    contiguous complex128) or of their (re, im) pairs."""
+    a = np.asarray(links)
+    if np.iscomplexobj(a):
+        return np.ascontiguousarray(a, dtype=np.complex128).view(np.float64)
+    return np.ascontiguousarray(a, dtype=np.float64)
 
 
 def qcd_set_links(h, links) -> None:
-    a = np.asarray(links)
-    if np.iscomplexobj(a):
-        a = np.stack([a.real, a.imag], axis=-1)
-    a = np.ascontiguousarray(a, dtype=np.float64)
-    _check(lib().qcd_set_links(h, _dptr(a)))
+    _check(lib().qcd_set_links(h, _dptr(_links_f64(links))))
 
 
 def qcd_link_bytes(h) -> int:
@@ -368,16 +373,13 @@ def qcd_batch_sweep(h, n: int, n_sweeps: int, n_overrelax: int, seed: int, measu
 
 
 def qcd_batch_get_links(h, index: int, V: int) -> np.ndarray:
-    out = np.empty((V, 4, 2, 2, 2), np.float64)
-    _check(lib().qcd_batch_get_links(h, index, _dptr(out)))
-    return out[..., 0] + 1j * out[..., 1]
+    out = np.empty((V, 4, 2, 2), np.complex128)
+    _check(lib().qcd_batch_get_links(h, index, _dptr(out.view(np.float64))))
+    return out
 
 
 def qcd_batch_set_links(h, index: int, links) -> None:
-    a = np.asarray(links)
-    if np.iscomplexobj(a):
-        a = np.stack([a.real, a.imag], axis=-1)
-    _check(lib().qcd_batch_set_links(h, index, _dptr(np.ascontiguousarray(a, dtype=np.float64))))
+    _check(lib().qcd_batch_set_links(h, index, _dptr(_links_f64(links))))
 
 
 def qcd_batch_get_sweep(h) -> int:
