@@ -908,10 +908,10 @@ __device__ __forceinline__ void final_sums(const double* const (&p)[N], const in
 // Warps per series for the longest series' length.
 inline int final_warps(int n) { return std::max(1, std::min(6, (n + 127) / 128)); }
 
-// out = {P, P_s, P_t, Re L, Im L} of the measurement's block partials; one thread
-// per number (one FP64 division each).
+// out = {P, P_s, P_t, Re L, Im L} of the measurement's block partials times their
+// scales; one thread per number (one FP64 division each).
 static __global__ void __launch_bounds__(FINAL_THREADS)
-    measure_final_kernel(const Ctx a, int n_plaq_blocks, int n_poly_blocks, double poly_scale) {
+    measure_final_kernel(const Ctx a, int n_plaq_blocks, int n_poly_blocks, double plaq_scale, double poly_scale) {
   __shared__ double sh[4][8];
   const double* q = a.partials + 2 * int64_t(n_plaq_blocks);
   final_sums<4>({a.partials, a.partials + 1, q, q + 1}, {n_plaq_blocks, n_plaq_blocks, n_poly_blocks, n_poly_blocks},
@@ -919,9 +919,14 @@ static __global__ void __launch_bounds__(FINAL_THREADS)
   if (threadIdx.x < 5) {
     const double V = 2.0 * double(a.g.Vh), V3 = double(a.g.Ns) * a.g.Ns * a.g.Ns;
     const int t = threadIdx.x;
-    const double num = t == 0 ? sh[0][0] + sh[1][0] : t < 3 ? sh[t - 1][0] : sh[t - 1][0] * poly_scale;
-    a.meas_out[t] = num / (t == 0 ? 6.0 * V : t < 3 ? 3.0 * V : V3);
+    const double num = t == 0 ? sh[0][0] + sh[1][0] : sh[t - 1][0];
+    a.meas_out[t] = num * (t < 3 ? plaq_scale : poly_scale) / (t == 0 ? 6.0 * V : t < 3 ? 3.0 * V : V3);
   }
+}
+
+inline void launch_measure_final(const Ctx& a, cudaStream_t st, int np, int nl, double plaq_scale,
+                                 double poly_scale) {
+  measure_final_kernel<<<1, 32 * 4 * final_warps(std::max(np, nl)), 0, st>>>(a, np, nl, plaq_scale, poly_scale);
 }
 
 // Final sums of a working sweep's fused measurement: the plaquette partials
@@ -1059,7 +1064,7 @@ cudaError_t launch_measure(const Ctx& a, int effective, cudaStream_t st) {
       default: measure_kernel<P, 2><<<np + nl, MEAS_THREADS, 0, st>>>(a, np); break;
     }
   }
-  measure_final_kernel<<<1, 32 * 4 * final_warps(std::max(np, nl)), 0, st>>>(a, np, nl, P::N == 3 ? 1.0 / 3.0 : 1.0);
+  launch_measure_final(a, st, np, nl, 1.0, P::N == 3 ? 1.0 / 3.0 : 1.0);
   return cudaGetLastError();
 }
 

@@ -630,6 +630,23 @@ inline bool su3c_split(const GeomH& g) { return (g.Vh + 31) / 32 <= 800; }
 // Links of one CTA for a block size of the caller.
 inline int su3c_links_per_cta(const GeomH& g, int block) { return su3c_split(g) ? 32 : block; }
 
+// Tr of the ordered product over t of the t-links of spatial site s0 = x + Ns (y + Ns z).
+__device__ __forceinline__ void su3c_poly_site(const Ctx& a, int site, SumF (&v)[2]) {
+  const int Ns = a.g.Ns, V3 = Ns * Ns * Ns;
+  const int xyz = site % Ns + site / Ns % Ns + site / (Ns * Ns);
+  Rows2 l = su3c_load(a.links, a.g, 3, xyz & 1, site >> 1);
+#pragma unroll 1
+  for (int t = 1; t < a.g.Nt; ++t)
+    l = su3c_mul(l, su3c_full(su3c_load(a.links, a.g, 3, (xyz + t) & 1, int((site + (long long)t * V3) >> 1))));
+  const Cx<float> l22 = cross2(l.e[0][0], l.e[1][1], l.e[0][1], l.e[1][0]);
+  v[0].add(l.e[0][0].re);
+  v[0].add(l.e[1][1].re);
+  v[0].add(l22.re);
+  v[1].add(l.e[0][0].im);
+  v[1].add(l.e[1][1].im);
+  v[1].add(l22.im);
+}
+
 // Polyakov loop of a working sweep's fused measurement: Tr of the
 // ordered product over t of the t-links of each spatial site, one thread per
 // site, products formed by rows 0-1 with row 2 rebuilt as for every FP32 link
@@ -639,26 +656,71 @@ inline int su3c_links_per_cta(const GeomH& g, int block) { return su3c_split(g) 
 // slower, 0.094 / 0.127 ms, and so did unrolling the t-loop by 4, 0.091 ms).
 // Block partials of Re and Im in a fixed order.
 static __global__ void __launch_bounds__(MEAS_THREADS) su3c_poly_kernel(const Ctx a) {
-  const long long V3 = (long long)a.g.Ns * a.g.Ns * a.g.Ns;
   const long long site = (long long)blockIdx.x * MEAS_THREADS + threadIdx.x;
   SumF v[2];
-  if (site < V3) {
-    const int Ns = a.g.Ns;
-    const int x = int(site % Ns), y = int((site / Ns) % Ns), z = int(site / ((long long)Ns * Ns));
-    const int s0 = x + Ns * (y + Ns * z), xyz = x + y + z;
-    Rows2 l = su3c_load(a.links, a.g, 3, xyz & 1, s0 >> 1);
-#pragma unroll 1
-    for (int t = 1; t < a.g.Nt; ++t)
-      l = su3c_mul(l, su3c_full(su3c_load(a.links, a.g, 3, (xyz + t) & 1, int((s0 + (long long)t * V3) >> 1))));
-    const Cx<float> l22 = cross2(l.e[0][0], l.e[1][1], l.e[0][1], l.e[1][0]);
-    v[0].add(l.e[0][0].re);
-    v[0].add(l.e[1][1].re);
-    v[0].add(l22.re);
-    v[1].add(l.e[0][0].im);
-    v[1].add(l.e[1][1].im);
-    v[1].add(l22.im);
+  if (site < (long long)a.g.Ns * a.g.Ns * a.g.Ns) su3c_poly_site(a, int(site), v);
+  block_sums(v, a.partials + 2 * blockIdx.x);
+}
+
+// Re Tr of the plaquette of plane (MU, NU) at x, of parity p (the final sums take the
+// 1/3: as an FP32 factor it shifted every plaquette by 3e-8 of itself): with
+// P = (Ut_mu(x) Ut_nu(x+mu)) (Ut_nu(x) Ut_mu(x+nu))^+ in SU(3), the upper 2x2 block of
+// P and its cofactor, Tr P = P00 + P11 + conj(P00 P11 - P01 P10).
+template <int FIELD, int MU, int NU>
+__device__ __forceinline__ float su3c_plaquette(const Ctx& a, int p, const LexSite& x) {
+  const Rows2 ab = su3c_mul(su3c_eff<FIELD, MU>(a, p, x), su3c_full(su3c_eff<FIELD, NU>(a, p ^ 1, lex_step<MU, +1>(a.g, x))));
+  const Rows2 dc = su3c_mul(su3c_eff<FIELD, NU>(a, p, x), su3c_full(su3c_eff<FIELD, MU>(a, p ^ 1, lex_step<NU, +1>(a.g, x))));
+  Cx<float> P[2][2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      XY s = xy_first(ab.e[i][0], dc.e[j][0]);
+      xy_add(s, ab.e[i][1], dc.e[j][1]);
+      xy_add(s, ab.e[i][2], dc.e[j][2]);
+      P[i][j] = xy_conj(s);
+    }
+  const Cx<float> c = cross2(P[0][0], P[1][1], P[0][1], P[1][0]);
+  return P[0][0].re + P[1][1].re + c.re;
+}
+
+// Plaquettes and Polyakov loop of a configuration, as measure_kernel, by two-row
+// products plane by plane.  Bound: the FMA pipes and the gather's latency (24 links
+// a site, 4 from memory); at 80 registers (some spills) 24 warps an SM hide more of
+// it than the generic kernel's 16, which kept U_mu(x) for three planes in full
+// matrices: measurement at 64^3x16 623 -> 443 us (0.26 of HBM; 64 / 72 / 96 / 128 registers:
+// 725 / 504 / 504 / 469), 48^3x16 287 -> 193, 20^3x6 31.5 -> 23.1.
+template <int FIELD>
+__global__ void __maxnreg__(80) su3c_measure_kernel(const Ctx a, int n_plaq_blocks) {
+  SumF v[2];
+  if (int(blockIdx.x) < n_plaq_blocks) {
+    // half of the block on either parity of the same sites
+    const int p = threadIdx.x / (MEAS_THREADS / 2), h = blockIdx.x * (MEAS_THREADS / 2) + threadIdx.x % (MEAS_THREADS / 2);
+    if (h < a.g.Vh) {
+      const LexSite x = lex_site_ytz(a.g, p, h);
+      v[0].add(su3c_plaquette<FIELD, 0, 1>(a, p, x));
+      v[0].add(su3c_plaquette<FIELD, 0, 2>(a, p, x));
+      v[0].add(su3c_plaquette<FIELD, 1, 2>(a, p, x));
+      v[1].add(su3c_plaquette<FIELD, 0, 3>(a, p, x));
+      v[1].add(su3c_plaquette<FIELD, 1, 3>(a, p, x));
+      v[1].add(su3c_plaquette<FIELD, 2, 3>(a, p, x));
+    }
+  } else {
+    const long long site = (long long)(int(blockIdx.x) - n_plaq_blocks) * MEAS_THREADS + threadIdx.x;
+    if (site < (long long)a.g.Ns * a.g.Ns * a.g.Ns) polyakov_site<SU3Policy<float>>(a, site, v[0], v[1]);
   }
   block_sums(v, a.partials + 2 * blockIdx.x);
+}
+
+inline cudaError_t su3c_launch_measure(const Ctx& a, int effective, cudaStream_t st) {
+  const int np = meas_plaq_blocks(a.g), nl = meas_poly_blocks(a.g);
+  switch (effective ? su3_field_level(a) : 0) {
+    case 0: su3c_measure_kernel<0><<<np + nl, MEAS_THREADS, 0, st>>>(a, np); break;
+    case 1: su3c_measure_kernel<1><<<np + nl, MEAS_THREADS, 0, st>>>(a, np); break;
+    default: su3c_measure_kernel<2><<<np + nl, MEAS_THREADS, 0, st>>>(a, np); break;
+  }
+  launch_measure_final(a, st, np, nl, 1.0 / 3.0, 1.0 / 3.0);
+  return cudaGetLastError();
 }
 
 inline cudaError_t su3c_measure_fused_tail(const Ctx& a, int block, cudaStream_t st) {

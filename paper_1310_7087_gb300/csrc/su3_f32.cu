@@ -11,7 +11,7 @@ const PolicyOps kOpsSU3F32 = PolicyOps{3,
                                        &su3c_launch_phase,
                                        &launch_reunit<SU3F>,
                                        &launch_start<SU3F>,
-                                       &launch_measure<SU3F>,
+                                       &su3c_launch_measure,
                                        &launch_to_canonical<SU3F>,
                                        &launch_from_canonical<SU3F>,
                                        &launch_set_frozen<SU3F>,
