@@ -444,18 +444,25 @@ __global__ void __launch_bounds__(96 * SPLIT, SU3D_CTAS / SPLIT)
   }
 }
 
-// Polyakov loop of a working sweep's fused measurement: three warps per 32 spatial
-// sites, warp r with row r of the running product over t; each converts row r of
-// the next link for the three.  FP64 block partials of Tr, in a fixed order.
-// (The plane sums, this kernel and the final sums add 41 us to a sweep of 16^3x4 and
-// 77 to one of 32^3x8; the separate FP64 measurement took 128 and 780.)
-static __global__ void __launch_bounds__(96) su3d_poly_kernel(const __grid_constant__ Ctx a) {
-  __shared__ FxTile tile[2][3][3];
-  __shared__ uint32_t flag[3][32];
-  __shared__ double sum[3][2];
-  const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
+// Three warps with 32 sites; the sums of Re and Im Tr over the warp's lanes.
+struct Su3dMeasTiles {
+  FxTile t[2][3][3];
+  uint32_t flag[3][32];
+};
+
+// FP64 for sites out of the fixed-point range, out of line.
+static __device__ __noinline__ double2 su3d_poly_fp64(const Ctx& a, int site) {
+  SumD v0, v1;
+  polyakov_site<SU3Policy<double>>(a, site, v0, v1);
+  return make_double2(v0.s, v1.s);
+}
+
+// Polyakov loop of 32 spatial sites: warp r with row r of the running product over
+// t; each converts row r of the next link for the three.
+__device__ __forceinline__ void su3d_poly(const Ctx& a, int base, Su3dMeasTiles& sh, int role, int lane, int bar,
+                                          double& re, double& im) {
   const int Ns = a.g.Ns, V3 = Ns * Ns * Ns;
-  const int site = blockIdx.x * 32 + lane, s0 = min(site, V3 - 1);
+  const int site = base + lane, s0 = min(site, V3 - 1);
   const int xyz = s0 % Ns + s0 / Ns % Ns + s0 / (Ns * Ns);
   const double2* links = reinterpret_cast<const double2*>(a.links) + 6 * a.g.plane;
   auto row = [&](int t) {
@@ -471,27 +478,32 @@ static __global__ void __launch_bounds__(96) su3d_poly_kernel(const __grid_const
     su3d_convert<1>(next, false, w, big);
     if (t + 1 < a.g.Nt) next = row(t + 1);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) tile[t & 1][role][k].put(lane, w[k]);
-    __syncthreads();  // (the other buffer's readers passed this one's predecessor)
+    for (int k = 0; k < 3; ++k) sh.t[t & 1][role][k].put(lane, w[k]);
+    bar_96(bar);  // (the other buffer's readers passed this one's predecessor)
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
       FxDot<false> d;
 #pragma unroll
-      for (int k = 0; k < 3; ++k) d.add(v[k], tile[t & 1][k][j].get(lane));
+      for (int k = 0; k < 3; ++k) d.add(v[k], sh.t[t & 1][k][j].get(lane));
       w[j] = d.limbs(bad);
     }
 #pragma unroll
     for (int k = 0; k < 3; ++k) v[k] = w[k];
   }
-  flag[role][lane] = (bad & FX_BAD) | (big & FX_BIG);
-  __syncthreads();
-  const bool in = site < V3, out_of_range = flag[0][lane] | flag[1][lane] | flag[2][lane];
+  sh.flag[role][lane] = (bad & FX_BAD) | (big & FX_BIG);
+  bar_96(bar);
+  const bool in = site < V3, out_of_range = sh.flag[0][lane] | sh.flag[1][lane] | sh.flag[2][lane];
   const FxC d = role == 0 ? v[0] : role == 1 ? v[1] : v[2];
   const bool fixed = in && !out_of_range;
-  double re = fx_warp_sum(fixed ? fx_value(d.re) : 0), im = fx_warp_sum(fixed ? fx_value(d.im) : 0);
+  re = fx_warp_sum(fixed ? fx_value(d.re) : 0);
+  im = fx_warp_sum(fixed ? fx_value(d.im) : 0);
   if (role == 0 && __any_sync(0xffffffffu, in && out_of_range)) {
     SumD v0, v1;
-    if (in && out_of_range) polyakov_site<SU3Policy<double>>(a, site, v0, v1);
+    if (in && out_of_range) {
+      const double2 v = su3d_poly_fp64(a, site);
+      v0.s = v.x;
+      v1.s = v.y;
+    }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
       v0.merge_down(off);
@@ -500,6 +512,18 @@ static __global__ void __launch_bounds__(96) su3d_poly_kernel(const __grid_const
     re += v0.s;
     im += v1.s;
   }
+}
+
+// Polyakov loop of a working sweep's fused measurement, 32 spatial sites per CTA.
+// FP64 block partials of Tr, in a fixed order.  (The plane sums, this kernel and the
+// final sums add 41 us to a sweep of 16^3x4 and 77 to one of 32^3x8; the separate
+// FP64 measurement took 128 and 780.)
+static __global__ void __launch_bounds__(96) su3d_poly_kernel(const __grid_constant__ Ctx a) {
+  __shared__ Su3dMeasTiles sh;
+  __shared__ double sum[3][2];
+  const int lane = threadIdx.x & 31, role = threadIdx.x >> 5;
+  double re, im;
+  su3d_poly(a, blockIdx.x * 32, sh, role, lane, 1, re, im);
   if (lane == 0) {
     sum[role][0] = re;
     sum[role][1] = im;
@@ -559,10 +583,11 @@ inline cudaError_t su3d_launch_level(const Ctx& a, int parity, int mu, cudaStrea
   }
 }
 
-// Heat-bath and the reunitarizing overrelaxation are compiled in translation
-// units of their own.
+// Heat-bath, the reunitarizing overrelaxation and what measures are compiled in
+// translation units of their own.
 cudaError_t su3d_launch_hb(const Ctx& a, int parity, int mu, cudaStream_t st);
 cudaError_t su3d_launch_or_reunit(const Ctx& a, int parity, int mu, cudaStream_t st);
 cudaError_t su3d_launch_or_meas(const Ctx& a, int parity, int mu, cudaStream_t st);
+cudaError_t su3d_launch_measure(const Ctx& a, int effective, cudaStream_t st);
 
 }  // namespace qcd

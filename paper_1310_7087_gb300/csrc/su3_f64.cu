@@ -1,7 +1,7 @@
 // su3_f64.cu -- kernels of the gauge sweep for SU(3) with FP64 18-real links.
-// The phase update uses the fixed-point kernel of qcd_su3d.cuh;
-// reunitarization, start, measurements and layout conversion use the shared
-// templates.
+// The phase update and the measurements use the fixed-point kernels of
+// qcd_su3d.cuh and su3_f64_meas.cu; reunitarization, start and layout conversion use
+// the shared templates.
 #include "qcd_su3d.cuh"
 
 namespace qcd {
@@ -26,7 +26,7 @@ const PolicyOps kOpsSU3F64 = PolicyOps{3,
                                        &launch_phase,
                                        &launch_reunit<SU3D>,
                                        &launch_start<SU3D>,
-                                       &launch_measure<SU3D>,
+                                       &su3d_launch_measure,
                                        &launch_to_canonical<SU3D>,
                                        &launch_from_canonical<SU3D>,
                                        &launch_set_frozen<SU3D>,

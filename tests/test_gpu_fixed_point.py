@@ -83,3 +83,20 @@ def test_su3_working_sweep_measurement(q, Ns, Nt, flux, flux8, kind):
     assert np.abs(got - np.array(p + l)).max() < 1e-13
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("kind", ["unitary", "scaled"])
+@pytest.mark.parametrize("group,Ns,Nt,flux,flux8", [(3, 6, 2, 1, 0), (3, 10, 4, 1, 1), (2, 6, 2, 0, 0), (2, 10, 4, 2, 0)])
+def test_measurement(q, group, Ns, Nt, flux, flux8, kind):
+    """Ragged blocks, fields, and links out of the fixed-point range (their sites in
+    FP64) against the oracle: sums of 10^3 to 10^4 terms of the size of the largest."""
+    lat = q.Lattice(group, Ns, Nt, 5.7, flux, FP64_PLAIN, HOT, 7, flux8=flux8)
+    orc = oracle.OracleLattice(group, Ns, Nt, 5.7, flux, 10, 0, flux8=flux8)
+    start = links_of(kind, lat.get_links(), np.random.default_rng(3))
+    lat.set_links(start)
+    orc.set_links(start)
+    (p, l), (op, ol) = lat.measure(), orc.measure()
+    for got, ref in ((p, op), (l, ol), (lat.measure_bare(), orc.measure_bare())):
+        size = 1.0 if kind == "unitary" else 100.0 ** Nt
+        assert np.abs(np.array(got) - np.array(ref)).max() < 1e-12 * size, (got, ref)
+    lat.close()
