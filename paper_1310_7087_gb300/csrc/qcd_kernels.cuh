@@ -908,10 +908,11 @@ __device__ __forceinline__ void final_sums(const double* const (&p)[N], const in
 // Warps per series for the longest series' length.
 inline int final_warps(int n) { return std::max(1, std::min(6, (n + 127) / 128)); }
 
-// out = {P, P_s, P_t, Re L, Im L} of the measurement's block partials times their
-// scales; one thread per number (one FP64 division each).
+// out = {P, P_s, P_t, Re L, Im L} of the measurement's block partials over what
+// they are multiples of (N for sums of Re Tr; a factor 1/3 in double would be a
+// second rounding); one thread per number (one FP64 division each).
 static __global__ void __launch_bounds__(FINAL_THREADS)
-    measure_final_kernel(const Ctx a, int n_plaq_blocks, int n_poly_blocks, double plaq_scale, double poly_scale) {
+    measure_final_kernel(const Ctx a, int n_plaq_blocks, int n_poly_blocks, double plaq_n, double poly_n) {
   __shared__ double sh[4][8];
   const double* q = a.partials + 2 * int64_t(n_plaq_blocks);
   final_sums<4>({a.partials, a.partials + 1, q, q + 1}, {n_plaq_blocks, n_plaq_blocks, n_poly_blocks, n_poly_blocks},
@@ -920,13 +921,12 @@ static __global__ void __launch_bounds__(FINAL_THREADS)
     const double V = 2.0 * double(a.g.Vh), V3 = double(a.g.Ns) * a.g.Ns * a.g.Ns;
     const int t = threadIdx.x;
     const double num = t == 0 ? sh[0][0] + sh[1][0] : sh[t - 1][0];
-    a.meas_out[t] = num * (t < 3 ? plaq_scale : poly_scale) / (t == 0 ? 6.0 * V : t < 3 ? 3.0 * V : V3);
+    a.meas_out[t] = num / ((t < 3 ? plaq_n : poly_n) * (t == 0 ? 6.0 * V : t < 3 ? 3.0 * V : V3));
   }
 }
 
-inline void launch_measure_final(const Ctx& a, cudaStream_t st, int np, int nl, double plaq_scale,
-                                 double poly_scale) {
-  measure_final_kernel<<<1, 32 * 4 * final_warps(std::max(np, nl)), 0, st>>>(a, np, nl, plaq_scale, poly_scale);
+inline void launch_measure_final(const Ctx& a, cudaStream_t st, int np, int nl, double plaq_n, double poly_n) {
+  measure_final_kernel<<<1, 32 * 4 * final_warps(std::max(np, nl)), 0, st>>>(a, np, nl, plaq_n, poly_n);
 }
 
 // Final sums of a working sweep's fused measurement: the plaquette partials
@@ -934,10 +934,10 @@ inline void launch_measure_final(const Ctx& a, cudaStream_t st, int np, int nl, 
 // 3; `grid` block partials each) and the Polyakov-loop partials (nl pairs at
 // poly_offset).  Writes meas_out = {P, P_s, P_t, Re L, Im L, P_1, P_2, P_3}, P_mu the
 // mean plaquette of the planes phase mu sums: (y,x); (z,x), (z,y); (t,x), (t,y),
-// (t,z).  plane_scale multiplies the plane sums: 1 when the phase kernels summed
-// (1/N) Re Tr, 1/N when they summed Re Tr; poly_scale the Polyakov loop.
+// (t,z).  plane_n divides the plane sums: 1 when the phase kernels summed
+// (1/N) Re Tr, N when they summed Re Tr; poly_n the Polyakov loop.
 static __global__ void __launch_bounds__(FINAL_THREADS)
-    fused_final_kernel(const Ctx a, int grid, double plane_scale, int nl, int poly_offset, double poly_scale) {
+    fused_final_kernel(const Ctx a, int grid, double plane_n, int nl, int poly_offset, double poly_n) {
   __shared__ double sh[5][8];
   const double* pl = a.partials + poly_offset;
   final_sums<5>({a.partials + fused_plaq_offset(a.g, 1), a.partials + fused_plaq_offset(a.g, 2),
@@ -949,13 +949,13 @@ static __global__ void __launch_bounds__(FINAL_THREADS)
     const double sp = sh[0][0] + sh[1][0];
     const double num = t == 0 ? sp + sh[2][0] : t == 1 ? sp : t == 2 ? sh[2][0] : t < 5 ? sh[t][0] : sh[t - 5][0];
     const double den = t == 0 ? 6.0 * V : t < 3 || t == 7 ? 3.0 * V : t < 5 ? V3 : t == 5 ? V : 2.0 * V;
-    a.meas_out[t] = num * (t == 3 || t == 4 ? poly_scale : plane_scale) / den;
+    a.meas_out[t] = num / ((t == 3 || t == 4 ? poly_n : plane_n) * den);
   }
 }
-inline void launch_fused_final(const Ctx& a, cudaStream_t st, int grid, double plane_scale, int nl, int poly_offset,
-                               double poly_scale) {
+inline void launch_fused_final(const Ctx& a, cudaStream_t st, int grid, double plane_n, int nl, int poly_offset,
+                               double poly_n) {
   const int block = 32 * 5 * final_warps(std::max(grid, nl));
-  fused_final_kernel<<<1, block, 0, st>>>(a, grid, plane_scale, nl, poly_offset, poly_scale);
+  fused_final_kernel<<<1, block, 0, st>>>(a, grid, plane_n, nl, poly_offset, poly_n);
 }
 
 // ---------------------------------------------------------------------------
@@ -1051,20 +1051,13 @@ cudaError_t launch_set_frozen(const Ctx& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+// SU(2); SU(3) storages bring their own kernels.
 template <class P>
 cudaError_t launch_measure(const Ctx& a, int effective, cudaStream_t st) {
   const int np = meas_plaq_blocks(a.g), nl = meas_poly_blocks(a.g);
-  if constexpr (P::N == 2) {
-    if (effective && phases_on_links(a)) measure_kernel<P, 1><<<np + nl, MEAS_THREADS, 0, st>>>(a, np);
-    else measure_kernel<P, 0><<<np + nl, MEAS_THREADS, 0, st>>>(a, np);
-  } else {
-    switch (effective ? su3_field_level(a) : 0) {
-      case 0: measure_kernel<P, 0><<<np + nl, MEAS_THREADS, 0, st>>>(a, np); break;
-      case 1: measure_kernel<P, 1><<<np + nl, MEAS_THREADS, 0, st>>>(a, np); break;
-      default: measure_kernel<P, 2><<<np + nl, MEAS_THREADS, 0, st>>>(a, np); break;
-    }
-  }
-  launch_measure_final(a, st, np, nl, 1.0, P::N == 3 ? 1.0 / 3.0 : 1.0);
+  if (effective && phases_on_links(a)) measure_kernel<P, 1><<<np + nl, MEAS_THREADS, 0, st>>>(a, np);
+  else measure_kernel<P, 0><<<np + nl, MEAS_THREADS, 0, st>>>(a, np);
+  launch_measure_final(a, st, np, nl, 1.0, 1.0);
   return cudaGetLastError();
 }
 

@@ -719,14 +719,13 @@ inline cudaError_t su3c_launch_measure(const Ctx& a, int effective, cudaStream_t
     case 1: su3c_measure_kernel<1><<<np + nl, MEAS_THREADS, 0, st>>>(a, np); break;
     default: su3c_measure_kernel<2><<<np + nl, MEAS_THREADS, 0, st>>>(a, np); break;
   }
-  launch_measure_final(a, st, np, nl, 1.0 / 3.0, 1.0 / 3.0);
+  launch_measure_final(a, st, np, nl, 3.0, 3.0);
   return cudaGetLastError();
 }
 
 inline cudaError_t su3c_measure_fused_tail(const Ctx& a, int block, cudaStream_t st) {
   su3c_poly_kernel<<<meas_poly_blocks(a.g), MEAS_THREADS, 0, st>>>(a);
-  launch_fused_final(a, st, int(grid_for(a.g.Vh, su3c_links_per_cta(a.g, block))), 1.0 / 3.0, meas_poly_blocks(a.g), 0,
-                     1.0 / 3.0);
+  launch_fused_final(a, st, int(grid_for(a.g.Vh, su3c_links_per_cta(a.g, block))), 3.0, meas_poly_blocks(a.g), 0, 3.0);
   return cudaGetLastError();
 }
 

@@ -10,14 +10,15 @@
 // update itself goes by columns: the subgroup rotations mix rows, so warp c
 // rotates column c; the three rotations are found by one warp each.
 //
-// Bound: the integer pipe (ncu at 32^3x6: ALU 52 %, 21,200 warp instructions per
-// 32 updates, 18,000 of them the 12 + 1 products and their conversions; waits on
-// it and on dispatch are the largest stalls) where the FP64 form was bound by
-// the FP64 unit (94 % busy).  Overrelaxation / heat-bath phase, us, FP64 form ->
-// this: 4^3x4 73.8 / 118.9 -> 12 / 18; 16^3x4 75.8 / 126.2 -> 18 / 25; 32^3x8
-// 447 / 710 -> 149 / 215; 48^3x16 2868 / 4314 -> 915 / 1408.  One thread per
-// link (168 registers) took 1231 us for the last, with the matrices unrolled
-// for both kinds of staple 1665 (instruction cache).
+// Bound: the integer pipes (ncu at 32^3x8: widening multiply-adds and moves keep
+// the multiplier's pipe 61 % busy, adds, shifts and logic the ALU 51 %; 21,200
+// warp instructions per 32 updates; fixed-latency waits and the pipes' are the
+// largest stalls) where the FP64 form was bound by the FP64 unit (94 % busy).
+// Overrelaxation / heat-bath phase, us, FP64 form -> this: 4^3x4 73.8 / 118.9 ->
+// 12 / 18; 16^3x4 75.8 / 126.2 -> 18 / 25; 32^3x8 447 / 710 -> 149 / 215; 48^3x16
+// 2868 / 4314 -> 915 / 1408.  One thread per link (168 registers) took 1231 us for
+// the last, with the matrices unrolled for both kinds of staple 1665 (instruction
+// cache); one copy of the subgroup rotation for all three 1 to 2 % more.
 #pragma once
 
 #include <type_traits>
@@ -537,7 +538,7 @@ static __global__ void __launch_bounds__(96) su3d_poly_kernel(const __grid_const
 inline cudaError_t su3d_measure_fused_tail(const Ctx& a, int /*block*/, cudaStream_t st) {
   const int nl = fused_poly32_blocks(a.g);
   su3d_poly_kernel<<<nl, 96, 0, st>>>(a);
-  launch_fused_final(a, st, (a.g.Vh + 31) / 32, 1.0 / 3.0, nl, fused_plaq_offset(a.g, 4), 1.0 / 3.0);
+  launch_fused_final(a, st, (a.g.Vh + 31) / 32, 3.0, nl, fused_plaq_offset(a.g, 4), 3.0);
   return cudaGetLastError();
 }
 

@@ -101,7 +101,7 @@ __device__ __forceinline__ void su3d_plaquettes(const Ctx& a, int p, int base, S
 
 // Measurement of a configuration: CTAs of eight groups of three warps, 256 sites (as
 // measure_kernel's blocks, for the same partials): plaquettes, then the Polyakov loop.
-// Measurement at 16^3x4 / 32^3x8 / 48^3x16, us: 61 / 346 / 2226, against 128 / 772 /
+// Measurement at 16^3x4 / 32^3x8 / 48^3x16, us: 60 / 340 / 2190, against 128 / 772 /
 // 4880 by the FP64 kernel (SU(2), one thread a site: 24 / 66 / 396 against 42 / 159 / 898).
 template <int FIELD>
 __global__ void __launch_bounds__(768) su3d_measure_kernel(const __grid_constant__ Ctx a, int n_plaq_blocks) {
@@ -122,10 +122,12 @@ __global__ void __launch_bounds__(768) su3d_measure_kernel(const __grid_constant
     sum[warp][1] = v1;
   }
   __syncthreads();
-  if (threadIdx.x < 2) {
-    double r = 0.0;
-    for (int w = 0; w < 24; ++w) r += sum[w][threadIdx.x];
-    a.partials[2 * int64_t(blockIdx.x) + threadIdx.x] = r;
+  if (warp == 0) {  // a tree: 5 roundings on a path and 5 FP64 instructions instead of 23
+    const int g = 3 * ((lane >> 1) & 7), k = lane & 1;
+    double r = sum[g][k] + sum[g + 1][k] + sum[g + 2][k];
+#pragma unroll
+    for (int off = 8; off > 1; off >>= 1) r += __shfl_down_sync(0xffffffffu, r, off);
+    if (lane < 2) a.partials[2 * int64_t(blockIdx.x) + lane] = r;
   }
 }
 
@@ -137,7 +139,7 @@ inline cudaError_t su3d_launch_measure_field(const Ctx& a, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   const int np = meas_plaq_blocks(a.g), nl = meas_poly_blocks(a.g);
   su3d_measure_kernel<FIELD><<<np + nl, 768, bytes, st>>>(a, np);
-  launch_measure_final(a, st, np, nl, 1.0 / 3.0, 1.0 / 3.0);
+  launch_measure_final(a, st, np, nl, 3.0, 3.0);
   return cudaGetLastError();
 }
 
