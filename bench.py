@@ -41,13 +41,16 @@ UNIT = "link updates/s"
 # same direction, V/2 read + V/2 written, for V/2 updates per phase).
 LINK_BYTES = {(3, 1): 48, (3, 0): 144, (2, 1): 16, (2, 0): 32}
 TRANSFERS_PER_UPDATE = 9
-# FP64 flops of one SU(3) overrelaxation update in the FP64 kernel (FMA = 2):
-# staple 12 full 3x3 complex products (324 complex multiply-adds), W = U A
-# (27), the three subgroup rotations of U and the first two of W (60), at 8
-# flops each = 3,288, plus ~150 for the projections, norms and quaternion
-# squares.  The peak it is held to is measured in the run (qcd_probe_fp64_rate:
-# FP64 FMA chains filling every SM, CUDA events); the nominal 1.25 TFLOP/s of
-# GB300 (152 SMs x 2 FP64 FMA per clock x 2 flops x 2.07 GHz) is the fallback.
+# The SU(3) FP64 overrelaxation update runs in fixed point on the integer pipe: a
+# real multiply-add is three 32 x 32 -> 64 bit integer multiply-adds, so the 12
+# matrix products of the staple, U A (27 complex multiply-adds each) and the
+# rotations (60) are 411 x 4 x 3 = 4,932 of them; the multiplier's pipe takes 64 a
+# clock and SM (62.9 measured by independent chains), and shares it with the
+# compiler's register moves.  The carries, shifts and conversions between them
+# keep the ALU pipe about as busy.  The same update by FP64 instructions is 3,438 flops (FMA = 2):
+# that rate is reported against the FP64 unit's measured peak
+# (qcd_probe_fp64_rate) as "times the FP64 unit".
+INT_OR_MADS, INT_MADS_PER_CLOCK_SM, SMS = 4932, 64, 152
 FP64_OR_FLOPS = 3438
 FP64_PEAK_TFLOPS_NOMINAL = 1.25
 
@@ -794,7 +797,7 @@ def main():
         ms64 = f0.elapsed_time(f1) / n64
         pm, pn = q.qcd_get_profile(lat64.h)
         extras["fp64_plain"] = {"value": lu_per_step / (ms64 / 1e3), "unit": UNIT, "ms_per_step": ms64,
-                                "storage": "FP64 18-real", "bound": "fp64 alu",
+                                "storage": "FP64 18-real", "bound": "integer alu (fixed-point products)",
                                 "kernel_ms_per_step": {n: round(m / n64, 3) for n, m in zip(names, pm)},
                                 "fp32_speedup": (lu_per_step * args.steps / (t_ms / 1e3)) /
                                                 (lu_per_step / (ms64 / 1e3))}
@@ -805,11 +808,15 @@ def main():
                 peak64, src64 = q.qcd_probe_fp64_rate(stream) / 1e12, "measured in this run (qcd_probe_fp64_rate)"
             except q.QcdError as e:
                 peak64, src64 = FP64_PEAK_TFLOPS_NOMINAL, "nominal GB300 FP64 (probe failed: %s)" % e
+            mads = INT_OR_MADS * (w.volume // 2) / (or_ms / 1e3) / 1e12
+            peak_mads = INT_MADS_PER_CLOCK_SM * SMS * 2.07e9 / 1e12
             extras["fp64_plain"]["roofline"] = {
-                "bound": "alu", "kernel": "overrelax_phase", "unit": "TFLOP/s", "achieved": tf,
-                "peak": peak64, "frac": tf / peak64, "flops_per_update": FP64_OR_FLOPS,
-                "avg_launch_ms": or_ms, "peak_source": src64,
-                "nominal_peak": FP64_PEAK_TFLOPS_NOMINAL}
+                "bound": "alu", "kernel": "overrelax_phase", "unit": "T integer multiply-adds/s",
+                "achieved": mads, "peak": peak_mads, "frac": mads / peak_mads,
+                "avg_launch_ms": or_ms, "peak_source": "64 per clock and SM at 2.07 GHz, 152 SMs",
+                "fp64_flops_per_update": FP64_OR_FLOPS, "fp64_tflops_equivalent": tf,
+                "fp64_unit_tflops": peak64, "times_the_fp64_unit": tf / peak64, "fp64_unit_source": src64,
+                "fp64_unit_nominal": FP64_PEAK_TFLOPS_NOMINAL}
         lat64.close()
 
         extras["batched"] = run_batched(q, stream, world, rank, dist, workloads.batch_scan().sweeps)
