@@ -13,9 +13,11 @@
 //
 // Storage: one 16-byte vector per site and parity (FP32: float4; FP64: two
 // double2 planes), even/odd halves, components beyond N kept zero.
+#include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <limits>
 #include <new>
 #include <vector>
 
@@ -36,6 +38,7 @@ struct OnCtx {
   int N;
   int nhit;
   double kappa, lambda, delta;
+  float kf;  // 2 kappa for the FP32 test; NaN: every test in FP64
   uint32_t k0, k1;
   const uint32_t* sweep;
   uint32_t* sweep_rw;
@@ -185,7 +188,7 @@ struct OnHitsF64 {
   int K[4];
   __device__ __forceinline__ OnHitsF64(const OnCtx& a, const double phi[4], const double f[4])
       : two_kappa(2.0 * a.kappa), lambda(a.lambda), step(a.delta * 0x1p-23) {
-    kf = float(two_kappa);
+    kf = a.kf;
     lf = float(lambda);
     sf = float(step);
     df = fabsf(float(a.delta));
@@ -283,8 +286,8 @@ struct OnHits<double, N> : OnHitsF64<N> {
 
 // Blocks of up to 512 threads have to launch: 128 registers at most.  A sweep of
 // O(4) with 100 hits per site, us, before -> now: FP32 8^3x8 55.9 -> 49.8, 32^4
-// 456 -> 447 (80 registers; 64: 473, 128: 452); FP64 8^3x8 363 -> 85, 16^4 655 ->
-// 105, 32^4 8649 -> 873.  Bound: the integer pipe (1.25 Philox blocks per hit, 160
+// 456 -> 447 (80 registers; 64: 473, 128: 452); FP64 8^3x8 363 -> 81, 16^4 655 ->
+// 101, 32^4 8649 -> 822.  Bound: the integer pipe (1.25 Philox blocks per hit, 160
 // cycles of an SM sub-partition per warp and hit in FP32), at small sizes the
 // latency of one hit after another.
 constexpr int ON_MAXNREG_F32 = 80, ON_MAXNREG_F64 = 128;
@@ -502,6 +505,11 @@ OnCtx make_on_ctx(const qcd_on* L, uint64_t seed) {
   a.N = L->N;
   a.nhit = L->nhit;
   a.kappa = L->kappa;
+  // With steps or couplings this far from 1, underflow in FP32 could outgrow the
+  // test's bound of roundings.
+  a.kf = L->delta > 0x1p-60 && std::fabs(L->kappa) < 0x1p60 && std::fabs(L->lambda) < 0x1p60
+             ? float(2.0 * L->kappa)
+             : std::numeric_limits<float>::quiet_NaN();
   a.lambda = L->lambda;
   a.delta = L->delta;
   a.k0 = uint32_t(seed);  // lattice id 0

@@ -19,6 +19,7 @@ pytestmark = pytest.mark.gpu
     (4, 7, 0.3, 1e6, 1e-3, 1.0),     # a stiff constraint: the bound is loose
     (2, 5, -0.3, -1e-9, 0.8, 1.0),   # signs turned
     (4, 9, 0.3, 0.0, 1e45, 1e45),    # beyond FP32: every test in FP64
+    (4, 9, 0.3, 0.0, 1e-36, (1e-36, 1e36)),  # even and odd sites: steps that FP32 cannot hold
 ])
 def test_fp64_hits(N, nhit, kappa, lam, delta, scale):
     torch = pytest.importorskip("torch")
@@ -30,13 +31,18 @@ def test_fp64_hits(N, nhit, kappa, lam, delta, scale):
     oracle.build()
     m = q.ONModel(N, 4, 6, kappa, lam, delta, FP64_PLAIN, HOT, 9, nhit=nhit)
     o = oracle.OracleON(N, 4, 6, kappa, lam, delta, nhit)
-    start = m.get_field() * scale
+    s = np.arange(4 ** 3 * 6)
+    odd = (s + s // 4 + s // 16 + s // 64) & 1
+    size = np.take(np.broadcast_to(scale, 2), odd)[:, None]
+    start = m.get_field() * size
     m.set_field(start)
     o.set_field(start)
     m.sweep(2, 9)
     o.sweep(2, 9)
     a, b = m.get_field(), o.get_field()
     assert m.accepted == o.accepted
-    assert np.abs(a - b).max() <= 1e-12 * max(1.0, np.abs(b).max())
+    for p in (0, 1):
+        w = odd == p
+        assert np.abs(a - b)[w].max() <= 1e-12 * max(size[w].max(), np.abs(b[w]).max())
     m.close()
     o.close()
