@@ -195,7 +195,9 @@ QCD_HD uint64_t fx_abs(int64_t v) { return v < 0 ? 0 - uint64_t(v) : uint64_t(v)
 
 // 1 / n for n in [1/4, 4) (2^58 units): a 24-bit seed y = 2^-27 yi (absolute
 // error below 2^-23 of it) and one step of third order, y (1 + e + e^2) with
-// e = 1 - n y formed exactly to 2^-58.
+// e = 1 - n y formed exactly to 2^-58.  At most 4 - 2^-58, the largest number that
+// two limbs hold: n = 1/4 is met exactly (one component of a normalised block), and
+// rounded down n may read a few units less where the norm is not below 1/4.
 QCD_HD int64_t fx_reciprocal(int64_t n) {
   const Fx l = fx_limbs(n);
   const float f = float(l.hi > 0 ? l.hi : 1);  // n 2^29
@@ -208,7 +210,9 @@ QCD_HD int64_t fx_reciprocal(int64_t n) {
   const int64_t e = fx_sub(int64_t(1) << FX_UNIT, prod);
   const int32_t es = int32_t(e >> 18);
   const int64_t t = e + (fx_mad(es, es, 0) >> 22);
-  return (int64_t(yi) << 31) + ((int64_t(yi) * (t >> 2)) >> 25);
+  const int64_t y = (int64_t(yi) << 31) + ((int64_t(yi) * (t >> 2)) >> 25);
+  constexpr int64_t top = (int64_t(1) << (FX_UNIT + 2)) - 1;
+  return y < top ? y : top;
 }
 
 // Left-normalises the quaternion w so that its largest component is in
@@ -240,6 +244,29 @@ QCD_HD bool fx_overrelax(int64_t w[4], Fx r[4]) {
     t.add(l[k], sl);
     const int64_t v = t.value() * 2;
     r[k] = fx_limbs(k == 0 ? v - (int64_t(1) << FX_UNIT) : -v);
+  }
+  return true;
+}
+
+// u <- V^+ u^+ V^+ = 2 <V^+, u> V^+ - u for the unit quaternion V = A / |A| (A of any
+// scale): the overrelaxation of an SU(2) link.  False, and u as it was, for A = 0.
+QCD_HD bool fx_reflect(int64_t A[4], Fx u[4], uint32_t& bad) {
+  if (!fx_normalise4(A)) return false;
+  Fx w[4];
+  FxAcc n, d;
+  for (int k = 0; k < 4; ++k) {
+    w[k] = fx_limbs(k ? -A[k] : A[k]);
+    n.add(w[k], w[k]);
+    d.add(w[k], u[k]);
+  }
+  FxAcc f;
+  f.add(fx_limbs(d.value()), fx_limbs(fx_reciprocal(n.value())));
+  fx_check(f.value(), bad);  // at most |u| / |A| with A normalised above 1/2
+  const Fx s = fx_limbs(f.value());
+  for (int k = 0; k < 4; ++k) {
+    FxAcc t;
+    t.add(w[k], s);
+    u[k] = fx_limbs(fx_sub(2 * t.value(), fx_value(u[k])));
   }
   return true;
 }

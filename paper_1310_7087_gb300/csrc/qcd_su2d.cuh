@@ -121,26 +121,7 @@ __device__ __forceinline__ double su2d_update(const Ctx& a, int parity, int mu, 
     su2d_load<false, CG>(a, mu, parity, x.s, u, big);
     if (phased) su2d_phase<false, false>(a, x.c[0], u, bad);
     if ((bad & FX_BAD) || (big & FX_BIG)) return su2d_general<FIELD, KIND, CG>(a, parity, mu, x, sweep);
-    // V^+ U^+ V^+ = 2 <V^+, U> V^+ - U for the unit quaternion V = A / |A|
-    if (fx_normalise4(A)) {
-      Fx w[4];
-      FxAcc n, d;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        w[k] = fx_limbs(k ? -A[k] : A[k]);
-        n.add(w[k], w[k]);
-        d.add(w[k], u[k]);
-      }
-      FxAcc f;
-      f.add(fx_limbs(d.value()), fx_limbs(fx_reciprocal(n.value())));
-      fx_check(f.value(), bad);  // at most |U| / |A| with A normalised above 1/2
-      const Fx s = fx_limbs(f.value());
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        FxAcc t;
-        t.add(w[k], s);
-        u[k] = fx_limbs(fx_sub(2 * t.value(), fx_value(u[k])));
-      }
+    if (fx_reflect(A, u, bad)) {
       if (bad & FX_BAD) return su2d_general<FIELD, KIND, CG>(a, parity, mu, x, sweep);
     } else {
       keep = true;

@@ -1,0 +1,113 @@
+"""The fixed-point arithmetic of the FP64 kernels (qcd_fix.cuh, qcd_fixmath.cuh) at
+the ends of its ranges, run by the host compiler against long double.  Bounds: a
+few units of 2^-58 per function, as in test_fixed_point (2^-54, and 2^-53 where a
+unit vector is squared)."""
+import os
+import platform
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1310_7087_gb300", "csrc")
+
+pytestmark = pytest.mark.skipif(platform.machine() not in ("x86_64", "aarch64"),
+                                reason="needs a long double wider than double")
+
+HEAD = r"""
+#include "qcd_fixmath.cuh"
+#include <cstdio>
+#include <random>
+using namespace qcd;
+typedef long double L;
+static const L U = (L)(1ll << 58), PI = 3.14159265358979323846264338327950288L;
+// the 24 units of the Hurwitz quaternions (the first 8: the quaternion group)
+static void hurwitz(int i, double q[4]) {
+  for (int k = 0; k < 4; ++k) q[k] = i < 8 ? (i >> 1) == k ? 1 - 2 * (i & 1) : 0.0 : 0.5 - ((i - 8) >> k & 1);
+}
+static int64_t units(double x) { return (int64_t)(x * (double)(1ll << 58)); }
+static Fx limbs(double x) { uint32_t b = 0; return fx_load(x, b); }
+"""
+
+
+def run(tmp_path, body):
+    src, exe = tmp_path / "fix.cpp", tmp_path / "fix"
+    src.write_text(HEAD + body)
+    subprocess.run(["g++", "-O2", "-I" + CSRC, "-x", "c++", str(src), "-o", str(exe)], check=True)
+    return subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split()
+
+
+def test_reciprocal_ends(tmp_path):
+    """1/n next to 1/4 and to 4, through the limbs that its users cut it into.  The
+    squared norm of a normalised block may read a few units below 1/4 (products
+    are rounded down) while the norm is not below it: 1/n is then within 2^-52 of 4."""
+    out = run(tmp_path, r"""
+int main() {
+  L err = 0, below = 0;
+  for (int64_t d = -16; d < 200000; ++d) {
+    for (int end = 0; end < 2; ++end) {
+      const int64_t n = end ? (int64_t(1) << 60) - 17 - d : (int64_t(1) << 56) + d;
+      const L y = fx_value(fx_limbs(fx_reciprocal(n))) / U;
+      if (!end && d < 0) below = fmaxl(below, fabsl(y - 4));
+      else err = fmaxl(err, fabsl(y * (n / U) - 1));
+    }
+  }
+  printf("%Lg %Lg\n", err, below);
+}
+""")
+    assert float(out[0]) < 2.0 ** -54 and float(out[1]) < 2.0 ** -52, out
+
+
+def test_overrelaxation_of_exact_blocks(tmp_path):
+    """The SU(3) subgroup rotation and the SU(2) reflection for staples that are a
+    multiple of a Hurwitz quaternion (cold links with centre elements among them) and
+    for a block with one large component."""
+    out = run(tmp_path, r"""
+int main() {
+  L rot = 0, refl = 0;
+  int bad_links = 0;
+  std::mt19937_64 g(1);
+  std::normal_distribution<double> z;
+  auto check = [&](const int64_t A[4]) {
+    L v[4], n2 = 0;
+    for (int k = 0; k < 4; ++k) { v[k] = A[k] / U; n2 += v[k] * v[k]; }
+    int64_t w[4] = {A[0], A[1], A[2], A[3]};
+    Fx r[4];
+    fx_overrelax(w, r);
+    for (int k = 0; k < 4; ++k)
+      rot = fmaxl(rot, fabsl(fx_value(r[k]) / U - (k ? -2 * v[0] * v[k] / n2 : 2 * v[0] * v[0] / n2 - 1)));
+    for (int i = 0; i < 40; ++i) {
+      double q[4], m = 0;
+      if (i < 24) hurwitz(i, q);
+      else {
+        for (int k = 0; k < 4; ++k) { q[k] = z(g); m += q[k] * q[k]; }
+        for (int k = 0; k < 4; ++k) q[k] /= sqrt(m);
+      }
+      Fx u[4];
+      L dot = 0;
+      for (int k = 0; k < 4; ++k) { u[k] = limbs(q[k]); w[k] = A[k]; dot += (k ? -v[k] : v[k]) * (fx_value(u[k]) / U); }
+      uint32_t bad = 0;
+      fx_reflect(w, u, bad);
+      if (bad & FX_BAD) { ++bad_links; continue; }
+      L e[4];
+      for (int k = 0; k < 4; ++k) e[k] = 2 * dot / n2 * (k ? -v[k] : v[k]) - (L)q[k];
+      for (int k = 0; k < 4; ++k) refl = fmaxl(refl, fabsl(fx_value(u[k]) / U - e[k]));
+    }
+  };
+  for (int i = 0; i < 24; ++i)
+    for (double s : {1.0, 2.0, 3.0, 4.0, 5.0, 6.0, 0.5, 0.25}) {
+      double q[4];
+      hurwitz(i, q);
+      const int64_t A[4] = {units(s * q[0]), units(s * q[1]), units(s * q[2]), units(s * q[3])};
+      check(A);
+    }
+  for (int p = 54; p < 61; ++p)
+    for (int m = 0; m < 32; ++m) {
+      int64_t A[4];
+      for (int k = 0; k < 4; ++k) A[k] = m >> k & 1 ? -1 : 0;
+      A[m & 3] = m & 16 ? -(int64_t(1) << p) : int64_t(1) << p;
+      check(A);
+    }
+  printf("%Lg %Lg %d\n", rot, refl, bad_links);
+}
+""")
+    assert float(out[0]) < 2.0 ** -53 and float(out[1]) < 2.0 ** -53 and out[2] == "0", out

@@ -1,0 +1,88 @@
+"""FP64 links at the ends of the fixed-point range, each phase against the oracle:
+links that are centre elements, signs or elements of the quaternion group, whose
+staples are exact multiples of group elements (or vanish).  An update divides by the norm of a
+subgroup block, at least 1 among these unless it is 0, so FP64 rounding stays far below 1e-10."""
+import numpy as np
+import pytest
+
+import oracle
+from workloads import COLD, FP64_PLAIN
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def q():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_1310_7087_gb300 import build
+    build.build()
+    import paper_1310_7087_gb300 as q
+    oracle.build()
+    return q
+
+
+def exact_links(kind, group, V, rng):
+    """(V, 4, N, N) links: a few centre elements in a cold lattice, or random signs or random elements of a finite group."""
+    one = np.eye(group, dtype=complex)
+    if group == 2:
+        i, j = np.array([[1j, 0], [0, -1j]]), np.array([[0, 1], [-1, 0]], complex)
+        elements = np.array([one, i, j, i @ j])
+        elements = np.concatenate([elements, -elements])
+    else:
+        elements = np.array([np.diag(d) for d in ((1, 1, 1), (1, -1, -1), (-1, 1, -1), (-1, -1, 1))], complex)
+    links = np.broadcast_to(one, (V, 4, group, group)).copy()
+    if kind == "centre":  # the links around one see staples of 5 - 1; SU(3): diagonal signs
+        for s in range(0, V, 37):
+            links[s, s % 4] = -one if group == 2 else elements[1 + s % 3]
+    elif kind == "signs":
+        links *= rng.choice([1.0, -1.0], (V, 4))[:, :, None, None]
+    else:
+        links = elements[rng.integers(0, len(elements), (V, 4))]
+    return links
+
+
+def step(q, lat, orc, kind, parity, mu):
+    lat.phase(kind, parity, mu, 5)
+    if kind == q.QCD_OVERRELAX_REUNIT:
+        orc.phase(q.QCD_OVERRELAX, parity, mu, 5)
+        orc.reunitarize_phase(parity, mu)
+    else:
+        orc.phase(kind, parity, mu, 5)
+    return np.abs(lat.get_links() - orc.get_links()).max()
+
+
+@pytest.mark.parametrize("group,Ns,Nt,kind", [(2, 4, 4, "centre"), (2, 4, 4, "signs"), (2, 4, 4, "group"),
+                                              (2, 20, 6, "centre"), (2, 20, 6, "signs"), (2, 20, 6, "group"),
+                                              (3, 4, 4, "centre"), (3, 4, 4, "group"), (3, 18, 4, "group"),
+                                              (3, 20, 6, "centre"), (3, 20, 6, "group")])
+def test_overrelaxation_of_exact_links(q, group, Ns, Nt, kind):
+    lat = q.Lattice(group, Ns, Nt, 2.3, 0, FP64_PLAIN, COLD, 7)
+    orc = oracle.OracleLattice(group, Ns, Nt, 2.3, 0, 10, 0)
+    start = exact_links(kind, group, Ns ** 3 * Nt, np.random.default_rng(3))
+    for k, parity, mu in ((q.QCD_OVERRELAX, 0, 0), (q.QCD_OVERRELAX, 1, 3), (q.QCD_OVERRELAX_REUNIT, 1, 1)):
+        lat.set_links(start)
+        orc.set_links(start)
+        assert step(q, lat, orc, k, parity, mu) < 1e-10, (k, parity, mu)
+    lat.close()
+
+
+def test_batch_overrelaxation_of_exact_links(q):
+    """At a coupling where every heat-bath try fails the links reach the overrelaxation as they were set."""
+    Ns, Nt = [4, 6], [4, 2]
+    b = q.Batch(Ns, Nt, [1e-300] * 2, [0, 0], FP64_PLAIN, COLD, 5)
+    for i in range(2):
+        start = exact_links("centre" if i else "group", 2, Ns[i] ** 3 * Nt[i], np.random.default_rng(3))
+        b.set_links(i, start)
+        orc = oracle.OracleLattice(2, Ns[i], Nt[i], 1e-300, 0, 10, i)
+        orc.set_links(start)
+        orc.sweep(1, 1, 5)
+        if i == 0:
+            first = orc
+    got = b.sweep(1, 1, 5)
+    for i, o in enumerate((first, orc)):
+        assert np.abs(b.get_links(i) - o.get_links()).max() < 1e-10, i
+        p, l = o.measure()
+        np.testing.assert_allclose(got[i, 0], list(p) + list(l), atol=1e-12)
+    b.close()
