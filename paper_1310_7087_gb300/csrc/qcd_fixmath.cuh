@@ -117,15 +117,17 @@ QCD_HD void fx_sincos(uint32_t x, int64_t& c, int64_t& s) {
   if (quadrant >= 2) s = -s;
 }
 
-// 1 / sqrt(n) for n in [1/4, 4].
+// 1 / sqrt(n) for n in [1/4, 4].  The seed y stays below 2 (it can round up to it at
+// n = 1/4): y^2 has to fit two limbs, and one unit of 2^-27 is within the seed's error.
 QCD_HD int64_t fx_rsqrt(int64_t n) {
   const Fx l = fx_limbs(n);
   const float f = float(l.hi > 0 ? l.hi : 1);  // n 2^29
 #ifdef __CUDA_ARCH__
-  const int32_t yi = __float2int_rn(rsqrtf(f) * 3109888511975.f);  // 2^41.5 / sqrt(n 2^29) = y 2^27
+  const int32_t seed = __float2int_rn(rsqrtf(f) * 3109888511975.f);  // 2^41.5 / sqrt(n 2^29) = y 2^27
 #else
-  const int32_t yi = int32_t(3109888511975.f / std::sqrt(f) + 0.5f);
+  const int32_t seed = int32_t(3109888511975.f / std::sqrt(f) + 0.5f);
 #endif
+  const int32_t yi = seed < (1 << 28) ? seed : (1 << 28) - 1;
   const Fx y2 = fx_limbs(fx_mad(yi, yi, 0) << 4);
   FxAcc m;
   m.add(l, y2);
@@ -138,7 +140,7 @@ QCD_HD int64_t fx_rsqrt(int64_t n) {
 // sqrt(x) for x in [0, 4).
 QCD_HD int64_t fx_sqrt(int64_t x) {
   if (x <= 0) return 0;
-  const int k = (fx_clz(uint64_t(x)) - 5) >> 1;  // x 4^k in [1/4, 2)
+  const int k = (fx_clz(uint64_t(x)) - 5) >> 1;  // x 4^k in [1/2, 2)
   const int64_t n = k >= 0 ? int64_t(uint64_t(x) << (2 * k)) : x >> (-2 * k);
   const int64_t s = fx_product(n, fx_rsqrt(n));
   return k >= 0 ? s >> k : s << -k;

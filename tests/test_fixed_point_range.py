@@ -111,3 +111,20 @@ int main() {
 }
 """)
     assert float(out[0]) < 2.0 ** -53 and float(out[1]) < 2.0 ** -53 and out[2] == "0", out
+
+
+def test_rsqrt_ends(tmp_path):
+    """1/sqrt(n) next to 1/4 (where a rounded seed can reach 2, and rounded down n may
+    read a few units less) and to 4."""
+    out = run(tmp_path, r"""
+int main() {
+  L err = 0;
+  auto check = [&](int64_t n) { err = fmaxl(err, fabsl(fx_rsqrt(n) / U * sqrtl(n / U) - 1)); };
+  for (int64_t d = 0; d < 200000; ++d) { check((int64_t(1) << 56) + d); check((int64_t(1) << 60) - 1 - d); }
+  for (int64_t d = 1; d <= 16; ++d) check((int64_t(1) << 56) - d);
+  for (int p = 17; p < 36; ++p)
+    for (int64_t d = 0; d < 20000; ++d) check((int64_t(1) << 56) + (d << p) / 7);
+  printf("%Lg\n", err);
+}
+""")
+    assert float(out[0]) < 2.0 ** -54, out

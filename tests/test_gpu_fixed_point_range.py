@@ -38,7 +38,7 @@ def exact_links(kind, group, V, rng):
             links[s, s % 4] = -one if group == 2 else elements[1 + s % 3]
     elif kind == "signs":
         links *= rng.choice([1.0, -1.0], (V, 4))[:, :, None, None]
-    else:
+    elif kind == "group":
         links = elements[rng.integers(0, len(elements), (V, 4))]
     return links
 
@@ -65,6 +65,22 @@ def test_overrelaxation_of_exact_links(q, group, Ns, Nt, kind):
         lat.set_links(start)
         orc.set_links(start)
         assert step(q, lat, orc, k, parity, mu) < 1e-10, (k, parity, mu)
+    lat.close()
+
+
+@pytest.mark.parametrize("group,Ns,Nt,flux,kind", [(2, 4, 4, 0, "centre"), (2, 4, 4, 4, "cold"), (2, 2, 2, 1, "cold"),
+                                                   (2, 20, 6, 100, "cold"), (2, 4, 4, 0, "group"), (3, 4, 4, 0, "centre"),
+                                                   (3, 4, 4, 4, "cold"), (3, 18, 4, 0, "centre"), (3, 20, 6, 100, "cold")])
+def test_heatbath_of_exact_links(q, group, Ns, Nt, flux, kind):
+    """Field phases of a quarter turn from site to site (flux = Ns^2 / 4) make staples 4 and 2 of a cold lattice."""
+    lat = q.Lattice(group, Ns, Nt, 2.3, flux, FP64_PLAIN, COLD, 7)
+    orc = oracle.OracleLattice(group, Ns, Nt, 2.3, flux, 10, 0)
+    start = exact_links(kind, group, Ns ** 3 * Nt, np.random.default_rng(3))
+    for parity, mu in ((0, 0), (1, 1), (1, 3)):
+        lat.set_links(start)
+        orc.set_links(start)
+        assert step(q, lat, orc, q.QCD_HEATBATH, parity, mu) < 1e-10, (parity, mu)
+    assert lat.exhausted == orc.exhausted
     lat.close()
 
 
