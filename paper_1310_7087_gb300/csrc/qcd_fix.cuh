@@ -250,6 +250,9 @@ QCD_HD bool fx_overrelax(int64_t w[4], Fx r[4]) {
 
 // u <- V^+ u^+ V^+ = 2 <V^+, u> V^+ - u for the unit quaternion V = A / |A| (A of any
 // scale): the overrelaxation of an SU(2) link.  False, and u as it was, for A = 0.
+// u is read with components below 2; what a link off the group can take out of range
+// (the product with the normalised block reaches 2 |u|, the result |u|) is checked
+// before it is cut into limbs.
 QCD_HD bool fx_reflect(int64_t A[4], Fx u[4], uint32_t& bad) {
   if (!fx_normalise4(A)) return false;
   Fx w[4];
@@ -259,14 +262,19 @@ QCD_HD bool fx_reflect(int64_t A[4], Fx u[4], uint32_t& bad) {
     n.add(w[k], w[k]);
     d.add(w[k], u[k]);
   }
+  const int64_t dv = d.value();
+  fx_check(dv, bad);
   FxAcc f;
-  f.add(fx_limbs(d.value()), fx_limbs(fx_reciprocal(n.value())));
-  fx_check(f.value(), bad);  // at most |u| / |A| with A normalised above 1/2
-  const Fx s = fx_limbs(f.value());
+  f.add(fx_limbs(dv), fx_limbs(fx_reciprocal(n.value())));
+  const int64_t fv = f.value();  // at most |u| / |A| with A normalised above 1/2
+  fx_check(fv, bad);
+  const Fx s = fx_limbs(fv);
   for (int k = 0; k < 4; ++k) {
     FxAcc t;
     t.add(w[k], s);
-    u[k] = fx_limbs(fx_sub(2 * t.value(), fx_value(u[k])));
+    const int64_t v = fx_sub(2 * t.value(), fx_value(u[k]));
+    fx_check(v, bad);
+    u[k] = fx_limbs(v);
   }
   return true;
 }

@@ -128,7 +128,8 @@ __device__ __forceinline__ double su2d_update(const Ctx& a, int parity, int mu, 
     }
     if (keep && !reunit) return 0.0;
   }
-  if (phased) su2d_phase<false, true>(a, x.c[0], u, bad);  // Ut_new B^+
+  // Ut_new B^+ (components below 2 before, so below 4 = 2^60 and within two limbs after)
+  if (phased) su2d_phase<false, true>(a, x.c[0], u, bad);
   Quat<double> q;
   bool done = false;
   if (reunit) {

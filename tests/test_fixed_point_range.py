@@ -128,3 +128,43 @@ int main() {
 }
 """)
     assert float(out[0]) < 2.0 ** -54, out
+
+
+def test_reflection_of_links_off_the_group(tmp_path):
+    """Links whose components are below 2 but whose norm reaches 4: reflected to within
+    four times a unit link's bound, or reported as out of range."""
+    out = run(tmp_path, r"""
+int main() {
+  std::mt19937_64 g(2);
+  std::normal_distribution<double> z;
+  std::uniform_real_distribution<double> un(0.3, 4.0);
+  L err = 0;
+  long fixed = 0, unit_bad = 0;
+  for (long it = 0; it < 2000000; ++it) {
+    double a[4], q[4], na = 0, nq = 0;
+    for (int k = 0; k < 4; ++k) { a[k] = z(g); q[k] = z(g); na += a[k] * a[k]; nq += q[k] * q[k]; }
+    const double ra = un(g) * 1.5 / sqrt(na), rq = (it % 4 ? un(g) : 1.0) / sqrt(nq);
+    bool inside = true;
+    if (it % 3 == 0)  // a link along the staple's adjoint: the largest product
+      for (int k = 0; k < 4; ++k) q[k] = (k ? -1 : 1) * a[k] / sqrt(na) * sqrt(nq) + 0.05 * q[k];
+    Fx u[4];
+    int64_t w[4];
+    L v[4], n2 = 0, dot = 0;
+    for (int k = 0; k < 4; ++k) {
+      inside &= fabs(q[k] * rq) < 2;
+      w[k] = units(a[k] * ra); v[k] = w[k] / U; n2 += v[k] * v[k];
+    }
+    if (!inside) continue;
+    for (int k = 0; k < 4; ++k) { u[k] = limbs(q[k] * rq); dot += (k ? -v[k] : v[k]) * (fx_value(u[k]) / U); }
+    L e[4];
+    for (int k = 0; k < 4; ++k) e[k] = 2 * dot / n2 * (k ? -v[k] : v[k]) - fx_value(u[k]) / U;
+    uint32_t bad = 0;
+    fx_reflect(w, u, bad);
+    if (bad & FX_BAD) { unit_bad += it % 4 == 0 && it % 3; continue; }
+    ++fixed;
+    for (int k = 0; k < 4; ++k) err = fmaxl(err, fabsl(fx_value(u[k]) / U - e[k]));
+  }
+  printf("%Lg %ld %ld\n", err, fixed, unit_bad);
+}
+""")
+    assert float(out[0]) < 2.0 ** -51 and int(out[1]) > 500000 and out[2] == "0", out

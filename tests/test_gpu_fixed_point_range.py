@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 
 import oracle
-from workloads import COLD, FP64_PLAIN
+from workloads import COLD, FP64_PLAIN, HOT
 
 pytestmark = pytest.mark.gpu
 
@@ -81,6 +81,23 @@ def test_heatbath_of_exact_links(q, group, Ns, Nt, flux, kind):
         orc.set_links(start)
         assert step(q, lat, orc, q.QCD_HEATBATH, parity, mu) < 1e-10, (parity, mu)
     assert lat.exhausted == orc.exhausted
+    lat.close()
+
+
+@pytest.mark.parametrize("group,Ns,Nt,flux", [(2, 4, 4, 1), (2, 6, 6, 0), (2, 20, 6, 1), (3, 4, 4, 1), (3, 20, 6, 0)])
+def test_links_off_the_group(q, group, Ns, Nt, flux):
+    """A third of the links with norms of 1.2 to 4: components below 2 among them, their products and reflections
+    beyond it.  The bound is for links of norm 4."""
+    lat = q.Lattice(group, Ns, Nt, 2.3, flux, FP64_PLAIN, HOT, 7)
+    orc = oracle.OracleLattice(group, Ns, Nt, 2.3, flux, 10, 0)
+    start, rng = lat.get_links(), np.random.default_rng(3)
+    pick = rng.random(start.shape[:2]) < 1 / 3
+    start[pick] *= rng.uniform(1.2, 4.0, pick.sum())[:, None, None]
+    for kind, parity, mu in ((q.QCD_OVERRELAX, 0, 0), (q.QCD_OVERRELAX, 1, 1), (q.QCD_OVERRELAX_REUNIT, 0, 1),
+                             (q.QCD_HEATBATH, 0, 3)):
+        lat.set_links(start)
+        orc.set_links(start)
+        assert step(q, lat, orc, kind, parity, mu) < 4e-10, (kind, parity, mu)
     lat.close()
 
 
