@@ -12,7 +12,7 @@
 // 2^-54 of each FP64 rounding of a number in [1/2, 1); sums of products are
 // exact between the two.
 //
-// Ranges: for |v| < 2 a limb product is below 2^60 (hi hi') or 2^59 (hi lo'),
+// Ranges, above: for |v| < 2 a limb product is below 2^60 (hi hi') or 2^59 (hi lo'),
 // so a three-term complex dot product (6 real products per part, 12 cross
 // terms) stays below 2^62.6 in both accumulators.  fx_load reports the largest
 // exponent it saw and fx_check any result outside (-2, 2); a caller that finds
@@ -192,6 +192,19 @@ QCD_HD int fx_clz(uint64_t v) {
 #endif
 }
 QCD_HD uint64_t fx_abs(int64_t v) { return v < 0 ? 0 - uint64_t(v) : uint64_t(v); }
+// At least the largest |w_k|, below its next power of two.
+QCD_HD uint64_t fx_size4(const int64_t w[4]) { return fx_abs(w[0]) | fx_abs(w[1]) | fx_abs(w[2]) | fx_abs(w[3]); }
+
+// Whether every part of a staple sum of SU(2) links is below 2^-5 (relative errors
+// would pass 2^-50): two in 10^7 random sums of six unit quaternions.
+QCD_HD bool fx_small(const int64_t A[4]) { return (fx_size4(A) >> (FX_UNIT - 5)) == 0; }
+// The same for a subgroup block of U A / 8 (twice the block), U or A small: all below
+// 2^-8, one in 10^7 blocks of random links.
+QCD_HD bool fx_small_block(const int64_t w[4]) { return (fx_size4(w) >> (FX_UNIT - 8)) == 0; }
+// Collects the parts of a row or a quaternion; fx_tiny: all were below 1/4, which a unit
+// one's are not (1/2 of the largest of four, 0.4 of six).
+QCD_HD uint32_t fx_part(Fx v) { return uint32_t(v.hi ^ (v.hi >> 31)); }
+QCD_HD bool fx_tiny(uint32_t parts) { return (parts >> (FX_LIMB - 2)) == 0; }
 
 // 1 / n for n in [1/4, 4) (2^58 units): a 24-bit seed y = 2^-27 yi (absolute
 // error below 2^-23 of it) and one step of third order, y (1 + e + e^2) with
@@ -218,7 +231,7 @@ QCD_HD int64_t fx_reciprocal(int64_t n) {
 // Left-normalises the quaternion w so that its largest component is in
 // [1/2, 1); returns 0 for w = 0.
 QCD_HD bool fx_normalise4(int64_t w[4]) {
-  const uint64_t m = fx_abs(w[0]) | fx_abs(w[1]) | fx_abs(w[2]) | fx_abs(w[3]);
+  const uint64_t m = fx_size4(w);
   if (m == 0) return false;
   const int z = fx_clz(m) - 1;
   for (int k = 0; k < 4; ++k) w[k] = int64_t(uint64_t(w[k]) << z) >> 5;

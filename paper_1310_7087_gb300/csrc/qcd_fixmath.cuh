@@ -227,8 +227,7 @@ __device__ __forceinline__ FxKpFirst fx_kp_first(const Stream& tries, const Stre
 // all that follows are fixed point again.
 __device__ __forceinline__ bool fx_heatbath(int64_t w[4], double inv_scale, int nhit, const Stream& tries,
                                             const FxKpFirst& f, Fx r[4]) {
-  const uint64_t m = fx_abs(w[0]) | fx_abs(w[1]) | fx_abs(w[2]) | fx_abs(w[3]);
-  const int shift = fx_clz(m) - 6;  // |w| = |w 2^shift| 2^-shift
+  const int shift = fx_clz(fx_size4(w)) - 6;  // |w| = |w 2^shift| 2^-shift
   fx_normalise4(w);
   Fx v[4];
   FxAcc n;

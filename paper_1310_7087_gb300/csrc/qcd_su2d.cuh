@@ -100,11 +100,10 @@ __device__ __forceinline__ double su2d_update(const Ctx& a, int parity, int mu, 
   const bool phased = FIELD && mu == 1;
   using P = SU2Policy<double>;
   Fx u[4];
-  bool keep = false;
+  if ((bad & FX_BAD) || (big & FX_BIG) || fx_small(A)) return su2d_general<FIELD, KIND, CG>(a, parity, mu, x, sweep);
   if (KIND == KIND_HB) {
-    if ((bad & FX_BAD) || (big & FX_BIG)) return su2d_general<FIELD, KIND, CG>(a, parity, mu, x, sweep);
     const Stream dir = make_stream(a.k0, a.k1, uint32_t(x.s), sweep, mu, 0, KIND_DIR);
-    if (a.beta == 0.0 || (A[0] | A[1] | A[2] | A[3]) == 0) {
+    if (a.beta == 0.0) {
       const Quat<double> R = su2d_haar(dir);
       u[0] = fx_load(R.q0, big);
       u[1] = fx_load(R.q1, big);
@@ -119,14 +118,10 @@ __device__ __forceinline__ double su2d_update(const Ctx& a, int parity, int mu, 
     }
   } else {
     su2d_load<false, CG>(a, mu, parity, x.s, u, big);
+    const bool tiny = fx_tiny(fx_part(u[0]) | fx_part(u[1]) | fx_part(u[2]) | fx_part(u[3]));
     if (phased) su2d_phase<false, false>(a, x.c[0], u, bad);
-    if ((bad & FX_BAD) || (big & FX_BIG)) return su2d_general<FIELD, KIND, CG>(a, parity, mu, x, sweep);
-    if (fx_reflect(A, u, bad)) {
-      if (bad & FX_BAD) return su2d_general<FIELD, KIND, CG>(a, parity, mu, x, sweep);
-    } else {
-      keep = true;
-    }
-    if (keep && !reunit) return 0.0;
+    fx_reflect(A, u, bad);
+    if (tiny || (bad & FX_BAD) || (big & FX_BIG)) return su2d_general<FIELD, KIND, CG>(a, parity, mu, x, sweep);
   }
   // Ut_new B^+ (components below 2 before, so below 4 = 2^60 and within two limbs after)
   if (phased) su2d_phase<false, true>(a, x.c[0], u, bad);

@@ -117,9 +117,10 @@ struct Su3dMeasShared : Su3dShared<SPLIT> {
   double sum[3];
 };
 
-// The rotation of subgroup `sub` from its block in sh.w into sh.r; returns
-// whether all tries of a heat-bath failed.  Out of line: one copy for the three
-// subgroups.
+// The rotation of subgroup `sub` from its block in sh.w into sh.r; whether all tries
+// of a heat-bath failed, or the block is too small for fixed point.  Out of line: one
+// copy for the three subgroups.
+enum { SU3D_EXHAUSTED = 1, SU3D_SMALL = 2 };
 template <int KIND, int SPLIT>
 __device__ __noinline__ unsigned su3d_rotation(Su3dShared<SPLIT>& sh, int lane, int sub, double beta, int nhit,
                                                uint32_t k0, uint32_t k1, uint32_t site, uint32_t sweep, int mu) {
@@ -130,7 +131,7 @@ __device__ __noinline__ unsigned su3d_rotation(Su3dShared<SPLIT>& sh, int lane, 
                   fx_value(wij.re) - fx_value(wji.re), fx_value(wii.im) - fx_value(wjj.im)};
   Fx r[4] = {};
   bool keep = false;
-  unsigned exhausted = 0;
+  unsigned status = fx_small_block(w) ? SU3D_SMALL : 0;  // (then the FP64 path does the update)
   if (KIND == KIND_HB) {
     const Stream dir = make_stream(k0, k1, site, sweep, mu, sub, KIND_DIR);
     if (beta == 0.0 || (w[0] | w[1] | w[2] | w[3]) == 0) {
@@ -148,7 +149,7 @@ __device__ __noinline__ unsigned su3d_rotation(Su3dShared<SPLIT>& sh, int lane, 
       for (int k = 0; k < 3; ++k) f.d[k] = sh.first[sub][2 + k][lane];
       // alpha = (2/3) beta k
       keep = !fx_heatbath(w, 0.375 / beta, nhit, make_stream(k0, k1, site, sweep, mu, sub, KIND_TRY), f, r);
-      exhausted = keep;
+      if (keep) status |= SU3D_EXHAUSTED;
     }
   } else {
     keep = !fx_overrelax(w, r);
@@ -156,7 +157,7 @@ __device__ __noinline__ unsigned su3d_rotation(Su3dShared<SPLIT>& sh, int lane, 
 #pragma unroll
   for (int k = 0; k < 4; ++k) sh.r[k][lane] = make_int2(r[k].hi, r[k].lo);
   sh.keep[lane] = keep;
-  return exhausted;
+  return status;
 }
 
 __device__ __forceinline__ void bar_96(int id) { asm volatile("bar.sync %0, 96;" ::"r"(id) : "memory"); }
@@ -322,7 +323,7 @@ __global__ void __launch_bounds__(96 * SPLIT, SU3D_CTAS / SPLIT)
       U[i] = sh.z[0][i][role].get(lane);
     }
   }
-  unsigned exhausted = 0;
+  unsigned status = 0;
 #pragma unroll
   for (int sub = 0; sub < 3; ++sub) {
     const int i = sub == 1 ? 1 : 0;
@@ -333,7 +334,7 @@ __global__ void __launch_bounds__(96 * SPLIT, SU3D_CTAS / SPLIT)
     }
     bar_96(1);
     if (role == sub)
-      exhausted = su3d_rotation<KIND, SPLIT>(sh, lane, sub, a.beta, a.nhit, a.k0, a.k1, uint32_t(s0), sweep, mu);
+      status = su3d_rotation<KIND, SPLIT>(sh, lane, sub, a.beta, a.nhit, a.k0, a.k1, uint32_t(s0), sweep, mu);
     bar_96(1);
     if (!sh.keep[lane]) {
       Fx r[4];
@@ -357,6 +358,7 @@ __global__ void __launch_bounds__(96 * SPLIT, SU3D_CTAS / SPLIT)
     }
   }
 
+  if (status & SU3D_SMALL) bad |= FX_BAD;
   sh.flag[role][lane] = (bad & FX_BAD) | (big & FX_BIG);
   if (reunit) {
 #pragma unroll
@@ -369,7 +371,7 @@ __global__ void __launch_bounds__(96 * SPLIT, SU3D_CTAS / SPLIT)
   if (on && out_of_range) {
     if (role == 0) v64 = su3_update_fp64<double, FIELD, KIND>(a, parity, mu, h);
   } else if (on) {
-    if (exhausted) atomicAdd(a.exhausted, (unsigned long long)exhausted);
+    if (status & SU3D_EXHAUSTED) atomicAdd(a.exhausted, 1ull);
     if (!reunit) {
       double2* out = reinterpret_cast<double2*>(a.links);
 #pragma unroll
@@ -491,6 +493,10 @@ __device__ __forceinline__ void su3d_poly(const Ctx& a, int base, Su3dMeasTiles&
 #pragma unroll
     for (int k = 0; k < 3; ++k) v[k] = w[k];
   }
+  uint32_t parts = 0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) parts |= fx_part(v[k].re) | fx_part(v[k].im);
+  if (fx_tiny(parts)) bad |= FX_BAD;
   sh.flag[role][lane] = (bad & FX_BAD) | (big & FX_BIG);
   bar_96(bar);
   const bool in = site < V3, out_of_range = sh.flag[0][lane] | sh.flag[1][lane] | sh.flag[2][lane];

@@ -36,6 +36,7 @@ __device__ __forceinline__ void su2d_plaquettes(const Ctx& a, int p, int h, SumD
         fx_check(t[k], bad);
         ab[k] = fx_limbs(t[k]);
       }
+      if (fx_tiny(fx_part(ab[0]) | fx_part(ab[1]) | fx_part(ab[2]) | fx_part(ab[3]))) bad |= FX_BAD;
       load(nu, p, x.s, x.c[0], u);
       load(mu, p ^ 1, x.s + ahead(nu), x.c[0], w);
       fx_qmul(u, w, t);

@@ -63,6 +63,10 @@ __device__ __forceinline__ void su3d_plaquettes(const Ctx& a, int p, int base, S
       for (int k = 0; k < 3; ++k) d.add(u[k], sh.t[0][k][j].get(lane));
       ab[j] = d.limbs(bad);
     }
+    uint32_t parts = 0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) parts |= fx_part(ab[j].re) | fx_part(ab[j].im);
+    if (fx_tiny(parts)) bad |= FX_BAD;
     FxAcc t;
 #pragma unroll
     for (int j = 0; j < 3; ++j) {

@@ -119,3 +119,31 @@ def test_batch_overrelaxation_of_exact_links(q):
         p, l = o.measure()
         np.testing.assert_allclose(got[i, 0], list(p) + list(l), atol=1e-12)
     b.close()
+
+
+@pytest.mark.parametrize("scale", [0.3, 1e-3, 1e-6])
+@pytest.mark.parametrize("group,Ns,Nt,flux", [(2, 4, 4, 1), (2, 20, 6, 0), (3, 4, 4, 1), (3, 18, 4, 0), (3, 20, 6, 1)])
+def test_small_links(q, group, Ns, Nt, flux, scale):
+    """All links scaled: fixed point has no digits of its own for small numbers, so these take the FP64 path where
+    they would lose some.  Errors relative to the sizes; a hot lattice's blocks (6 terms of order 1) are at least
+    1e-4 of theirs."""
+    lat = q.Lattice(group, Ns, Nt, 2.3, flux, FP64_PLAIN, HOT, 7)
+    orc = oracle.OracleLattice(group, Ns, Nt, 2.3, flux, 10, 0)
+    start = lat.get_links() * scale
+    for kind, parity, mu in ((q.QCD_OVERRELAX, 0, 0), (q.QCD_OVERRELAX, 1, 1), (q.QCD_HEATBATH, 0, 3)):
+        lat.set_links(start)
+        orc.set_links(start)
+        err = step(q, lat, orc, kind, parity, mu)
+        # (the SU(2) heat-bath replaces the link by a unit one)
+        assert err < 1e-10 * (scale if kind == q.QCD_OVERRELAX or group == 3 else 1.0), (kind, parity, mu, err)
+    assert lat.exhausted == orc.exhausted
+    lat.set_links(start)
+    orc.set_links(start)
+    (p, l), (op, ol) = lat.measure(), orc.measure()
+    assert np.abs(np.array(p) - np.array(op)).max() < 1e-12 * scale ** 4, (p, op)
+    assert np.abs(np.array(l) - np.array(ol)).max() < 1e-12 * scale ** Nt, (l, ol)
+    lat.phase(q.QCD_OVERRELAX_REUNIT, 1, 2, 5)
+    orc.phase(q.QCD_OVERRELAX, 1, 2, 5)
+    orc.reunitarize_phase(1, 2)
+    assert np.abs(lat.get_links() - orc.get_links()).max() < 1e-10
+    lat.close()
