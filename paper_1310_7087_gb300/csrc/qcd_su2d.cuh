@@ -100,7 +100,7 @@ __device__ __forceinline__ double su2d_update(const Ctx& a, int parity, int mu, 
   const bool phased = FIELD && mu == 1;
   using P = SU2Policy<double>;
   Fx u[4];
-  if ((bad & FX_BAD) || (big & FX_BIG) || fx_small(A)) return su2d_general<FIELD, KIND, CG>(a, parity, mu, x, sweep);
+  bool general = (bad & FX_BAD) || (big & FX_BIG) || fx_small(A);
   if (KIND == KIND_HB) {
     const Stream dir = make_stream(a.k0, a.k1, uint32_t(x.s), sweep, mu, 0, KIND_DIR);
     if (a.beta == 0.0) {
@@ -109,14 +109,19 @@ __device__ __forceinline__ double su2d_update(const Ctx& a, int parity, int mu, 
       u[1] = fx_load(R.q1, big);
       u[2] = fx_load(R.q2, big);
       u[3] = fx_load(R.q3, big);
-    } else {
+      general = false;
+    } else if (!general) {
       const Stream tries = make_stream(a.k0, a.k1, uint32_t(x.s), sweep, mu, 0, KIND_TRY);
-      if (!fx_heatbath(A, 1.0 / a.beta, a.nhit, tries, *first, u)) {
+      const int status = fx_heatbath(A, 1.0 / a.beta, a.nhit, tries, *first, u);
+      if (status == FX_EXHAUSTED) {
         atomicAdd(a.exhausted, 1ull);
         return 0.0;  // the link stays as it is
       }
+      general = status == FX_SMALL_DRAW;
     }
+    if (general) return su2d_general<FIELD, KIND, CG>(a, parity, mu, x, sweep);
   } else {
+    if (general) return su2d_general<FIELD, KIND, CG>(a, parity, mu, x, sweep);
     su2d_load<false, CG>(a, mu, parity, x.s, u, big);
     const bool tiny = fx_tiny(fx_part(u[0]) | fx_part(u[1]) | fx_part(u[2]) | fx_part(u[3]));
     if (phased) su2d_phase<false, false>(a, x.c[0], u, bad);

@@ -118,9 +118,9 @@ struct Su3dMeasShared : Su3dShared<SPLIT> {
 };
 
 // The rotation of subgroup `sub` from its block in sh.w into sh.r; whether all tries
-// of a heat-bath failed, or the block is too small for fixed point.  Out of line: one
-// copy for the three subgroups.
-enum { SU3D_EXHAUSTED = 1, SU3D_SMALL = 2 };
+// of a heat-bath failed (FX_EXHAUSTED), or the block or the draw is too small for fixed
+// point (FX_SMALL_DRAW: the FP64 path does the update).  Out of line: one copy for the
+// three subgroups.
 template <int KIND, int SPLIT>
 __device__ __noinline__ unsigned su3d_rotation(Su3dShared<SPLIT>& sh, int lane, int sub, double beta, int nhit,
                                                uint32_t k0, uint32_t k1, uint32_t site, uint32_t sweep, int mu) {
@@ -131,7 +131,7 @@ __device__ __noinline__ unsigned su3d_rotation(Su3dShared<SPLIT>& sh, int lane, 
                   fx_value(wij.re) - fx_value(wji.re), fx_value(wii.im) - fx_value(wjj.im)};
   Fx r[4] = {};
   bool keep = false;
-  unsigned status = fx_small_block(w) ? SU3D_SMALL : 0;  // (then the FP64 path does the update)
+  unsigned status = fx_small_block(w) ? FX_SMALL_DRAW : 0;
   if (KIND == KIND_HB) {
     const Stream dir = make_stream(k0, k1, site, sweep, mu, sub, KIND_DIR);
     if (beta == 0.0 || (w[0] | w[1] | w[2] | w[3]) == 0) {
@@ -143,13 +143,13 @@ __device__ __noinline__ unsigned su3d_rotation(Su3dShared<SPLIT>& sh, int lane, 
       r[3] = fx_load(R.q3, e);
     } else {
       FxKpFirst f;
-      f.e = sh.first[sub][0][lane];
+      f.e = __longlong_as_double(sh.first[sub][0][lane]);
       f.a3 = sh.first[sub][1][lane];
 #pragma unroll
       for (int k = 0; k < 3; ++k) f.d[k] = sh.first[sub][2 + k][lane];
       // alpha = (2/3) beta k
-      keep = !fx_heatbath(w, 0.375 / beta, nhit, make_stream(k0, k1, site, sweep, mu, sub, KIND_TRY), f, r);
-      if (keep) status |= SU3D_EXHAUSTED;
+      status |= fx_heatbath(w, 0.375 / beta, nhit, make_stream(k0, k1, site, sweep, mu, sub, KIND_TRY), f, r);
+      keep = status & FX_EXHAUSTED;
     }
   } else {
     keep = !fx_overrelax(w, r);
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(96 * SPLIT, SU3D_CTAS / SPLIT)
     if (group == 0) {
       const FxKpFirst f = fx_kp_first(make_stream(a.k0, a.k1, uint32_t(s0), sweep, mu, role, KIND_TRY),
                                       make_stream(a.k0, a.k1, uint32_t(s0), sweep, mu, role, KIND_DIR));
-      sh.first[role][0][lane] = f.e;
+      sh.first[role][0][lane] = __double_as_longlong(f.e);
       sh.first[role][1][lane] = f.a3;
 #pragma unroll
       for (int k = 0; k < 3; ++k) sh.first[role][2 + k][lane] = f.d[k];
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(96 * SPLIT, SU3D_CTAS / SPLIT)
     }
   }
 
-  if (status & SU3D_SMALL) bad |= FX_BAD;
+  if (status & FX_SMALL_DRAW) bad |= FX_BAD;
   sh.flag[role][lane] = (bad & FX_BAD) | (big & FX_BIG);
   if (reunit) {
 #pragma unroll
@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(96 * SPLIT, SU3D_CTAS / SPLIT)
   if (on && out_of_range) {
     if (role == 0) v64 = su3_update_fp64<double, FIELD, KIND>(a, parity, mu, h);
   } else if (on) {
-    if (status & SU3D_EXHAUSTED) atomicAdd(a.exhausted, 1ull);
+    if (status & FX_EXHAUSTED) atomicAdd(a.exhausted, 1ull);
     if (!reunit) {
       double2* out = reinterpret_cast<double2*>(a.links);
 #pragma unroll

@@ -147,3 +147,18 @@ def test_small_links(q, group, Ns, Nt, flux, scale):
     orc.reunitarize_phase(1, 2)
     assert np.abs(lat.get_links() - orc.get_links()).max() < 1e-10
     lat.close()
+
+
+@pytest.mark.parametrize("beta", [30.0, 1e3, 1e5])
+@pytest.mark.parametrize("group,Ns,Nt", [(2, 4, 4), (2, 20, 6), (3, 4, 4), (3, 18, 4), (3, 20, 6)])
+def test_weak_coupling(q, group, Ns, Nt, beta):
+    """Heat-bath phases of a cold lattice (blocks of norm 6) up to weak coupling: a link is about ten FP64
+    operations on numbers of order 1 in the oracle for each subgroup (2^-53 each), a tenth of it here."""
+    lat = q.Lattice(group, Ns, Nt, beta, 0, FP64_PLAIN, COLD, 7)
+    orc = oracle.OracleLattice(group, Ns, Nt, beta, 0, 10, 0)
+    for parity, mu in ((0, 0), (1, 3)):
+        lat.set_links(exact_links("cold", group, Ns ** 3 * Nt, None))
+        orc.set_links(lat.get_links())
+        assert step(q, lat, orc, q.QCD_HEATBATH, parity, mu) < (4e-15 if group == 2 else 1.2e-14), (parity, mu)
+    assert lat.exhausted == orc.exhausted
+    lat.close()
