@@ -16,6 +16,7 @@
 
 #include "qcd_device.cuh"
 #include "qcd_internal.h"
+#include "qcd_sums.cuh"
 
 namespace qcd {
 
@@ -729,31 +730,7 @@ __global__ void set_frozen_kernel(const Ctx a) {
   P::store(a.links, a.g, mu, parity_of(x), lex(a.g, x) >> 1, u);
 }
 
-// ---------------------------------------------------------------------------
-// Sums.  FP64 runs at a small fraction of the FP32 rate (one FP64 add of a warp
-// takes 64 cycles, and so does a conversion), so FP32 terms are summed without it:
-// Knuth's error-free TwoSum, t + e = s + s' exactly, keeps the errors in c, and
-// s + c is formed in FP64 once per warp.  The sum keeps a relative error near
-// 2^-48 (the rounding of c), as an FP64 sum of the FP32 terms would.
-// ---------------------------------------------------------------------------
-struct SumF {
-  float s = 0.f, c = 0.f;
-  __device__ __forceinline__ void add(float v) {
-    const float t = s + v;
-    const float bp = t - s;
-    c += (s - (t - bp)) + (v - bp);
-    s = t;
-  }
-  __device__ __forceinline__ void merge_down(int off) {
-    const float so = __shfl_down_sync(0xffffffffu, s, off), co = __shfl_down_sync(0xffffffffu, c, off);
-    const float t = s + so;
-    const float bp = t - s;
-    const float e = (s - (t - bp)) + (so - bp);
-    s = t;
-    c += co + e;
-  }
-  __device__ __forceinline__ double value() const { return double(s) + double(c); }
-};
+// FP64 terms, with the interface of SumF (qcd_sums.cuh).
 struct SumD {
   double s = 0.0;
   __device__ __forceinline__ void add(double v) { s += v; }
