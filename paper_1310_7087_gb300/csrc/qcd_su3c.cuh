@@ -663,35 +663,37 @@ static __global__ void __launch_bounds__(MEAS_THREADS) su3c_poly_kernel(const Ct
 }
 
 // Re Tr of the plaquette of plane (MU, NU) at x, of parity p (the final sums take the
-// 1/3: as an FP32 factor it shifted every plaquette by 3e-8 of itself): with
-// P = (Ut_mu(x) Ut_nu(x+mu)) (Ut_nu(x) Ut_mu(x+nu))^+ in SU(3), the upper 2x2 block of
-// P and its cofactor, Tr P = P00 + P11 + conj(P00 P11 - P01 P10).
+// 1/3: as an FP32 factor it shifted every plaquette by 3e-8 of itself): the trace of
+// (Ut_mu(x) Ut_nu(x+mu)) (Ut_nu(x) Ut_mu(x+nu))^+ over all three rows, so that links
+// whose rows are not orthonormal count as they are.  (The third row's part as the
+// cofactor of the product's upper 2x2 block is cheaper, 446 against 553 us at 64^3x16,
+// and right for unitary links only.)
 template <int FIELD, int MU, int NU>
 __device__ __forceinline__ float su3c_plaquette(const Ctx& a, int p, const LexSite& x) {
-  const Rows2 ab = su3c_mul(su3c_eff<FIELD, MU>(a, p, x), su3c_full(su3c_eff<FIELD, NU>(a, p ^ 1, lex_step<MU, +1>(a.g, x))));
-  const Rows2 dc = su3c_mul(su3c_eff<FIELD, NU>(a, p, x), su3c_full(su3c_eff<FIELD, MU>(a, p ^ 1, lex_step<NU, +1>(a.g, x))));
-  Cx<float> P[2][2];
+  const M3<float> ab = su3c_mul3(su3c_full(su3c_eff<FIELD, MU>(a, p, x)),
+                                 su3c_full(su3c_eff<FIELD, NU>(a, p ^ 1, lex_step<MU, +1>(a.g, x))));
+  const M3<float> d = su3c_full(su3c_eff<FIELD, NU>(a, p, x));
+  const M3<float> c = su3c_full(su3c_eff<FIELD, MU>(a, p ^ 1, lex_step<NU, +1>(a.g, x)));
+  float2 t = make_float2(0.f, 0.f);
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
+  for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      XY s = xy_first(ab.e[i][0], dc.e[j][0]);
-      xy_add(s, ab.e[i][1], dc.e[j][1]);
-      xy_add(s, ab.e[i][2], dc.e[j][2]);
-      P[i][j] = xy_conj(s);
+    for (int j = 0; j < 3; ++j) {
+      XY s = xy_first(d.e[i][0], c.e[0][j]);
+      xy_add(s, d.e[i][1], c.e[1][j]);
+      xy_add(s, d.e[i][2], c.e[2][j]);
+      t = ffma2(v2(ab.e[i][j]), v2(xy_mul(s)), t);
     }
-  const Cx<float> c = cross2(P[0][0], P[1][1], P[0][1], P[1][0]);
-  return P[0][0].re + P[1][1].re + c.re;
+  return t.x + t.y;
 }
 
-// Plaquettes and Polyakov loop of a configuration, as measure_kernel, by two-row
-// products plane by plane.  Bound: the FMA pipes and the gather's latency (24 links
-// a site, 4 from memory); at 80 registers (some spills) 24 warps an SM hide more of
-// it than the generic kernel's 16, which kept U_mu(x) for three planes in full
-// matrices: measurement at 64^3x16 623 -> 443 us (0.26 of HBM; 64 / 72 / 96 / 128 registers:
-// 725 / 504 / 504 / 469), 48^3x16 287 -> 193, 20^3x6 31.5 -> 23.1.
+// Plaquettes and Polyakov loop of a configuration, as measure_kernel, plane by plane
+// from two-row links (the generic kernel kept U_mu(x) for three planes in full
+// matrices).  Bound: the FMA pipes and the gather's latency (24 links a site, 4 from
+// memory).  Measurement at 64^3x16 616 -> 553 us (0.21 of HBM; 80 / 96 / 112 registers: 725 /
+// 615 / 580), 48^3x16 276 -> 242, 24^3x6 35.5 -> 26, 20^3x6 24.4 -> 22.8.
 template <int FIELD>
-__global__ void __maxnreg__(80) su3c_measure_kernel(const Ctx a, int n_plaq_blocks) {
+__global__ void __maxnreg__(128) su3c_measure_kernel(const Ctx a, int n_plaq_blocks) {
   SumF v[2];
   if (int(blockIdx.x) < n_plaq_blocks) {
     // half of the block on either parity of the same sites
