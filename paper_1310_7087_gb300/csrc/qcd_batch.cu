@@ -266,11 +266,13 @@ __device__ void batch_run(const BatchArgs& b, int li, const BatchLat& L, int j) 
 #endif
 
 // FP64 links take the fixed-point update (12.6 -> 4.8 ms per sweep of the
-// 64-lattice scan): 128 registers (4.9 ms; 112 / 96 / 80 / 64: 5.1 / 5.6 / 6.4 / 7.0).
+// 64-lattice scan): 128 registers (4.9 ms; 112 / 96 / 80 / 64: 5.1 / 5.6 / 6.4 / 7.0),
+// and 64 where a wave has more lattices than CTAs of 128 are resident (each lattice
+// needs one: at 64 threads 1,216, with 64 registers 2,432).
 constexpr int BATCH_MAXNREG_F64 = 128;
 
-template <typename R>
-__global__ void __maxnreg__(sizeof(R) == 8 ? BATCH_MAXNREG_F64 : QCD_BATCH_MAXNREG) batch_kernel(const BatchArgs b) {
+template <typename R, int REGS>
+__global__ void __maxnreg__(REGS) batch_kernel(const BatchArgs b) {
   const int li = b.cta_lattice[blockIdx.x];
   const BatchLat L = b.lat[li];
   const int j = int(blockIdx.x) - L.g0;
@@ -316,6 +318,7 @@ struct qcd_batch {
   int block = 0;        // threads per CTA; 0 = autotune on the next sweep
   int per_sm = 0;       // resident CTAs per SM used (0 = as many as fit)
   int total_ctas = 0;   // largest grid over the waves
+  bool narrow = false;  // FP64: the kernel with fewer registers, for more resident CTAs
   size_t wave_budget = 0;            // link bytes per wave (0: one wave)
   std::vector<int> wave_l0;          // first lattice of each wave, then n
   std::vector<int> wave_cta0;        // first entry of each wave in the CTA map
@@ -354,15 +357,16 @@ int* d_error(qcd_batch* B) { return reinterpret_cast<int*>(B->d_small + 4); }
 int* d_error_where(qcd_batch* B) { return reinterpret_cast<int*>(B->d_small + 8); }
 unsigned long long* d_exhausted(qcd_batch* B) { return reinterpret_cast<unsigned long long*>(B->d_small + 16); }
 
-void (*batch_kernel_ptr(int precision))(BatchArgs) {
-  return precision == QCD_FP64_PLAIN ? qcd::batch_kernel<double> : qcd::batch_kernel<float>;
+void (*batch_kernel_ptr(const qcd_batch* B))(BatchArgs) {
+  if (B->precision != QCD_FP64_PLAIN) return qcd::batch_kernel<float, QCD_BATCH_MAXNREG>;
+  return B->narrow ? qcd::batch_kernel<double, QCD_BATCH_MAXNREG> : qcd::batch_kernel<double, qcd::BATCH_MAXNREG_F64>;
 }
 
 // Resident CTAs for a block size (cooperative launch needs all CTAs
 // resident), at most `per_sm_cap` per SM when that is > 0.
 int resident_ctas(qcd_batch* B, int block, int per_sm_cap) {
   int per_sm = 0, sms = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel_ptr(B->precision), block, 0) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel_ptr(B), block, 0) !=
           cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, B->device) != cudaSuccess) {
     cudaGetLastError();
@@ -461,8 +465,15 @@ void drop_batch_graphs(qcd_batch* B) {
 // Lay out the CTA groups of every wave for `block` threads (at most `per_sm`
 // CTAs per SM, 0 = as many as fit) and upload descriptors.
 int configure(qcd_batch* B, int block, int per_sm = 0) {
-  const int capacity = resident_ctas(B, block, per_sm);
   form_waves(B);
+  int lattices = 0;  // of the fullest wave
+  for (size_t w = 0; w + 1 < B->wave_l0.size(); ++w) lattices = std::max(lattices, B->wave_l0[w + 1] - B->wave_l0[w]);
+  B->narrow = false;
+  int capacity = resident_ctas(B, block, per_sm);
+  if (capacity < lattices && B->precision == QCD_FP64_PLAIN) {
+    B->narrow = true;
+    capacity = resident_ctas(B, block, per_sm);
+  }
   std::vector<int> map;
   B->wave_cta0.clear();
   B->wave_ctas.clear();
@@ -534,7 +545,7 @@ int enqueue(qcd_batch* B, const BatchArgs& a0, cudaStream_t st, bool advance) {
     BatchArgs a = a0;
     a.cta_lattice = B->d_cta + B->wave_cta0[w];
     void* params[] = {&a};
-    BATCH_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(batch_kernel_ptr(B->precision)),
+    BATCH_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(batch_kernel_ptr(B)),
                                            dim3(B->wave_ctas[w]), dim3(B->block), params, 0, st));
   }
   if (advance) {
