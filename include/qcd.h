@@ -263,7 +263,10 @@ int qcd_set_sweep(qcd_lattice *lat, uint32_t sweep);
 int qcd_get_exhausted(qcd_lattice *lat, unsigned long long *count);
 
 /* Launch shape: threads per block of the phase kernels (0 = autotune on the
- * next sweep; otherwise a multiple of 32 in [32, 1024]). */
+ * next sweep; otherwise a multiple of 32 in [32, 1024], at most what the
+ * storage's kernels launch with).  Kernels with a CTA shape of their own take
+ * the value and launch as they are, and are not tuned: FP64 SU(3); FP32 SU(3)
+ * of at most 51,200 sites; FP64 SU(2) of at most 32,768. */
 int qcd_set_block(qcd_lattice *lat, int threads);
 int qcd_get_block(const qcd_lattice *lat, int *threads);
 

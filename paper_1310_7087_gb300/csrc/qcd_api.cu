@@ -369,8 +369,10 @@ int autotune(qcd_lattice* L) {
       return QCD_OK;
     }
   }
+  // Nothing to time where the kernels have a CTA shape of their own; a split lattice may
+  // not fit a device scratch copy.
   const char* env = getenv("QCD_AUTOTUNE");
-  if ((env && env[0] == '0') || L->split) {  // a split lattice may not fit a device scratch copy
+  if ((env && env[0] == '0') || L->split || L->ops->own_shape(L->g)) {
     L->block = 128;
     return QCD_OK;
   }

@@ -130,6 +130,9 @@ struct PolicyOps {
   // Largest block the phase kernels of this storage can launch with (the
   // minimum over heat-bath / overrelaxation, with and without the field).
   int (*max_phase_block)();
+  // Whether the phase kernels have a CTA shape of their own on this lattice and take
+  // no block size (nothing to tune).
+  bool (*own_shape)(const GeomH&);
 };
 
 // Effective-link phases are applied only in field mode 0 with a field.

@@ -255,7 +255,8 @@ PolicyOps su2c_ops(int precision) {
                    &launch_from_canonical<P>,
                    &launch_set_frozen<P>,
                    &su2c_measure_fused_tail<R>,
-                   &su2c_max_phase_block<R>};
+                   &su2c_max_phase_block<R>,
+                   [](const GeomH&) { return false; }};
 }
 
 }  // namespace qcd

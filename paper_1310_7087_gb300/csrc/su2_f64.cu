@@ -106,5 +106,6 @@ const PolicyOps kOpsSU2F64 = PolicyOps{2,
                                        &launch_from_canonical<SU2D>,
                                        &launch_set_frozen<SU2D>,
                                        &measure_fused_tail,
-                                       &max_phase_block};
+                                       &max_phase_block,
+                                       &su2d_split};
 }  // namespace qcd

@@ -17,6 +17,7 @@ cudaError_t launch_phase(const Ctx& a, int kind, int parity, int mu, int /*block
 // Block sizes that qcd_set_block takes (those of the 96-register FP64 kernel
 // that this storage had; the CTA shape is part of the kernel now).
 int max_phase_block() { return 640; }
+bool own_shape(const GeomH&) { return true; }
 }  // namespace
 
 using SU3D = SU3Policy<double>;
@@ -31,5 +32,6 @@ const PolicyOps kOpsSU3F64 = PolicyOps{3,
                                        &launch_from_canonical<SU3D>,
                                        &launch_set_frozen<SU3D>,
                                        &su3d_measure_fused_tail,
-                                       &max_phase_block};
+                                       &max_phase_block,
+                                       &own_shape};
 }  // namespace qcd
