@@ -649,6 +649,11 @@ static bool fused_measure_available(const qcd_lattice* L) {
 static bool fused_measure_by_phase(const qcd_lattice* L) {
   return fused_measure_available(L) && !(L->group == 3 && L->precision == QCD_FP64_PLAIN);
 }
+static int not_by_phase() {
+  return set_error(QCD_ERR_NOT_SUPPORTED,
+                   "the fused measurement phase by phase needs FP32 SU(3) or SU(2) storage and the effective-link "
+                   "field mode (qcd_working_sweep and qcd_measure take every lattice)");
+}
 
 static int measure_impl(qcd_lattice* L, int effective, double* plaq, double* poly);
 
@@ -686,9 +691,7 @@ int qcd_phase(qcd_lattice* L, int kind, int parity, int mu, uint64_t seed) {
       return set_error(QCD_ERR_INVALID_ARG,
                        "QCD_OVERRELAX_MEASURE is a phase of odd parity with mu >= 1 (got parity %d, mu %d)",
                        parity, mu);
-    if (!fused_measure_by_phase(L))
-      return set_error(QCD_ERR_NOT_SUPPORTED,
-                       "the fused measurement needs FP32 SU(3) or SU(2) storage and the effective-link field mode");
+    if (!fused_measure_by_phase(L)) return not_by_phase();
   }
   if (int rc = use_device(L)) return rc;
   static const int kinds[4] = {qcd::KIND_HB, qcd::KIND_OR, qcd::KIND_OR_REUNIT, qcd::KIND_OR_MEAS};
@@ -699,9 +702,7 @@ int qcd_phase(qcd_lattice* L, int kind, int parity, int mu, uint64_t seed) {
 int qcd_measure_fused_finish(qcd_lattice* L, double* host_out) {
   if (int rc = check(L)) return rc;
   if (!host_out) return set_error(QCD_ERR_INVALID_ARG, "host_out is null");
-  if (!fused_measure_by_phase(L))
-    return set_error(QCD_ERR_NOT_SUPPORTED,
-                     "the fused measurement needs FP32 SU(3) or SU(2) storage and the effective-link field mode");
+  if (!fused_measure_by_phase(L)) return not_by_phase();
   if (int rc = use_device(L)) return rc;
   QCD_CUDA(L->ops->measure_fused_tail(make_ctx(L, L->seed), phase_block(L), L->stream));
   QCD_CUDA(cudaMemcpyAsync(host_out, L->d_meas, 8 * sizeof(double), cudaMemcpyDeviceToHost, L->stream));
