@@ -769,12 +769,6 @@ __device__ __forceinline__ void block_sums(Sum (&v)[N], double* out) {
   }
 }
 
-__device__ __forceinline__ void block_sum_f32(float v, double* out) {
-  SumF s[1];
-  s[0].s = v;
-  block_sums(s, out);
-}
-
 // ---------------------------------------------------------------------------
 // Measurements: plaquette (spatial / temporal split) and Polyakov loop.
 // Products in the storage precision, sums as above: per-thread value, warp

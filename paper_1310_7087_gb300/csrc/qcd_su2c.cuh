@@ -162,9 +162,9 @@ __global__ void su2c_phase_kernel(const Ctx a, int parity) {
 template <typename R, bool FIELD, int MU>
 __global__ void su2c_or_meas_kernel(const Ctx a, int parity) {
   const int h = blockIdx.x * blockDim.x + threadIdx.x;
-  R v = R(0);
-  if (h < a.g.Vh) v = su2c_update<R, FIELD, KIND_OR_MEAS, MU, false>(a, parity, h, 0u);
-  block_sum_f32(v, a.partials + fused_plaq_offset(a.g, MU) + blockIdx.x);
+  SumOf<R> v[1];
+  if (h < a.g.Vh) v[0].s = su2c_update<R, FIELD, KIND_OR_MEAS, MU, false>(a, parity, h, 0u);
+  block_sums(v, a.partials + fused_plaq_offset(a.g, MU) + blockIdx.x);
 }
 
 template <typename R>

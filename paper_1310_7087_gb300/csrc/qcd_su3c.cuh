@@ -489,7 +489,7 @@ template <int FIELD, int MU>
 __global__ void __maxnreg__(QCD_SU3_MEAS_MAXNREG) su3c_or_meas_kernel(const Ctx a, int parity) {
   pdl_launch_dependents();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  float v = 0.f;
+  SumF v[1];
   if (i < a.g.Vh) {
     const LexSite x = lex_site_ytz(a.g, parity, i);
     pdl_wait();
@@ -498,9 +498,9 @@ __global__ void __maxnreg__(QCD_SU3_MEAS_MAXNREG) su3c_or_meas_kernel(const Ctx 
     const M3<float> A = su3c_staple<FIELD, MU, true>(a, parity, x, &low);
     M3<float> U = su3c_update<FIELD, KIND_OR_MEAS>(a, parity, MU, h, x, A,
                                                    su3c_full(su3c_load(a.links, a.g, MU, parity, h)));
-    v = su3c_plane_sum<FIELD>(a, MU, x, U, low);
+    v[0].s = su3c_plane_sum<FIELD>(a, MU, x, U, low);
   }
-  block_sum_f32(v, a.partials + fused_plaq_offset(a.g, MU) + blockIdx.x);
+  block_sums(v, a.partials + fused_plaq_offset(a.g, MU) + blockIdx.x);
 }
 
 // Small lattices: six warps share 32 links (lane = link), each computes one staple;
