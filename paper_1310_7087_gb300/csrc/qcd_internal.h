@@ -79,6 +79,8 @@ struct Ctx {
 
 static_assert(sizeof(Ctx) <= 128, "kernel argument struct grew past 128 bytes");
 
+// SMs of the GPU that the launch rules by waves of CTAs were measured on.
+constexpr int GB300_SMS = 152;
 constexpr int MEAS_THREADS = 256;
 constexpr int FINAL_THREADS = 1024;
 

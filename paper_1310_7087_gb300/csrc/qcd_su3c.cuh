@@ -755,7 +755,7 @@ inline void su3c_launch_split(const Ctx& a, int parity, int mu, cudaStream_t st)
   // sweep); within one it places the next phase's CTAs on the SMs that are left
   // (4^3x4: 115 -> 136).
   const unsigned grid = grid_for(a.g.Vh, 32);
-  if (grid > 3 * 152) launch_programmatic(su3c_split_kernel<FIELD, KIND>, grid, 192, st, a, parity, mu);
+  if (grid > 3 * GB300_SMS) launch_programmatic(su3c_split_kernel<FIELD, KIND>, grid, 192, st, a, parity, mu);
   else su3c_split_kernel<FIELD, KIND><<<grid, 192, 0, st>>>(a, parity, mu);
 }
 

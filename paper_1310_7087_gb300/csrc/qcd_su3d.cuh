@@ -571,13 +571,11 @@ inline cudaError_t su3d_launch_one(const Ctx& a, int parity, int mu, cudaStream_
 // FP64 unit holds its warp for 64 cycles); at full occupancy Z's go to the FP64
 // unit, which is otherwise idle (32^3x8 overrelaxation 151 -> 146 us; X's or Y's
 // too: 149).
-constexpr int SU3D_SMS = 152;
-
 template <int FIELD, int KIND>
 inline cudaError_t su3d_launch_kind(const Ctx& a, int parity, int mu, cudaStream_t st) {
   const int groups = (a.g.Vh + 31) / 32;
-  if (groups <= SU3D_SMS) return su3d_launch_one<FIELD, KIND, 6, 7>(a, parity, mu, st);
-  if (groups <= 3 * SU3D_SMS) return su3d_launch_one<FIELD, KIND, 2, 7>(a, parity, mu, st);
+  if (groups <= GB300_SMS) return su3d_launch_one<FIELD, KIND, 6, 7>(a, parity, mu, st);
+  if (groups <= 3 * GB300_SMS) return su3d_launch_one<FIELD, KIND, 2, 7>(a, parity, mu, st);
   return su3d_launch_one<FIELD, KIND, 1, 3>(a, parity, mu, st);
 }
 
