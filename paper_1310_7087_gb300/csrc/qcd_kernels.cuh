@@ -737,6 +737,16 @@ struct SumD {
   __device__ __forceinline__ void merge_down(int off) { s += __shfl_down_sync(0xffffffffu, s, off); }
   __device__ __forceinline__ double value() const { return s; }
 };
+template <int N>
+__device__ __forceinline__ double warp_values(const SumD (&v)[N]) {
+  double r = v[0].s;
+#pragma unroll
+  for (int k = 1; k < N; ++k) {
+    const double s = __shfl_sync(0xffffffffu, v[k].s, 0);
+    if ((threadIdx.x & 31) == 3 * k) r = s;
+  }
+  return r;
+}
 template <typename R>
 struct SumOfT {
   using type = SumD;
@@ -758,14 +768,15 @@ __device__ __forceinline__ void block_sums(Sum (&v)[N], double* out) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v[k].merge_down(off);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0)
+  const double r = warp_values(v);
 #pragma unroll
-    for (int k = 0; k < N; ++k) sh[k][warp] = v[k].value();
+  for (int k = 0; k < N; ++k)
+    if (lane == 3 * k) sh[k][warp] = r;
   __syncthreads();
   if (threadIdx.x < N) {
-    double r = sh[threadIdx.x][0];
-    for (int w = 1; w < int(blockDim.x >> 5); ++w) r += sh[threadIdx.x][w];
-    out[threadIdx.x] = r;
+    double t = sh[threadIdx.x][0];
+    for (int w = 1; w < int(blockDim.x >> 5); ++w) t += sh[threadIdx.x][w];
+    out[threadIdx.x] = t;
   }
 }
 

@@ -608,15 +608,16 @@ __global__ void __launch_bounds__(192, 3) su3c_split_kernel(const Ctx a, int par
     for (int sub = 0; sub < 3; ++sub)
       first[sub] = {sh.first[sub][0][lane], sh.first[sub][1][lane], sh.first[sub][2][lane],
                     sh.first[sub][3][lane], sh.first[sub][4][lane], sh.first[sub][5][lane]};
-  SumF v;
+  SumF v[1];
   if (on) {
     const M3<float> U = su3c_update<FIELD, KIND>(a, parity, mu, x.s >> 1, x, A, su3c_full(own), first, sweep);
-    if (KIND == KIND_OR_MEAS) v.s = su3c_plane_sum<FIELD>(a, mu, x, U, low);
+    if (KIND == KIND_OR_MEAS) v[0].s = su3c_plane_sum<FIELD>(a, mu, x, U, low);
   }
   if (KIND == KIND_OR_MEAS) {
 #pragma unroll
-    for (int off2 = 16; off2 > 0; off2 >>= 1) v.merge_down(off2);
-    if (lane == 0) a.partials[fused_plaq_offset(a.g, mu) + blockIdx.x] = v.value();
+    for (int off2 = 16; off2 > 0; off2 >>= 1) v[0].merge_down(off2);
+    const double r = warp_values(v);
+    if (lane == 0) a.partials[fused_plaq_offset(a.g, mu) + blockIdx.x] = r;
   }
 }
 

@@ -54,3 +54,37 @@ def test_plaquettes(q, kind, Ns, Nt, flux, flux8):
     assert np.abs(np.array(got) - plaquettes(U, B)).max() < 1.2e-6 * size, got
     assert np.abs(np.array(lat.measure_bare()) - plaquettes(U, np.ones((Ns, 3)))).max() < 1.2e-6 * size
     lat.close()
+
+
+@pytest.mark.parametrize("group,Ns", [(2, 4), (2, 10), (3, 4), (3, 10)])
+def test_sums_of_exact_terms(q, group, Ns):
+    """Links of small integers times powers of two, whose plaquettes are exact in FP32 and spread over 2^50: their
+    sums are those of FP64, at most one rounding (2^-53 of the sum of magnitudes) in each of some ten steps."""
+    rng = np.random.default_rng(2)
+    Nt, V = 2, Ns ** 3 * 2
+    k = rng.integers(-1, 2, (V, 4, 4 if group == 2 else 12)).astype(float)
+    if group == 2:
+        U = np.empty((V, 4, 2, 2), complex)
+        U[..., 0, 0], U[..., 0, 1] = k[..., 0] + 1j * k[..., 3], k[..., 2] + 1j * k[..., 1]
+        U[..., 1, 0], U[..., 1, 1] = -U[..., 0, 1].conj(), U[..., 0, 0].conj()
+    else:
+        U = np.zeros((V, 4, 3, 3), complex)
+        U[:, :, :2] = (k[..., ::2] + 1j * k[..., 1::2]).reshape(V, 4, 2, 3)
+    # SU(3): powers of the second row carry over to the third, so its links have one power for all
+    U *= 2.0 ** (rng.integers(-6, 7, (V, 4)) if group == 2 else np.full((V, 4), -1))[:, :, None, None]
+    lat = q.Lattice(group, Ns, Nt, 2.3, 0, FP32_COMPRESSED, HOT, 7)
+    lat.set_links(U)
+    U = lat.get_links().reshape(Nt, Ns, Ns, Ns, 4, group, group)
+    L, at, sums, sizes = [U[..., mu, :, :] for mu in range(4)], lambda f, mu: np.roll(f, -1, 3 - mu), [0, 0], [0, 0]
+    for mu in range(4):
+        for nu in range(mu + 1, 4):
+            ab, dc = L[mu] @ at(L[nu], mu), L[nu] @ at(L[mu], nu)
+            t = [int(v) for v in np.rint((ab * dc.conj()).real.sum((-1, -2)) * 2.0 ** 60).ravel()]
+            sums[nu == 3] += sum(t)
+            sizes[nu == 3] += sum(abs(v) for v in t)
+    P, S = np.array(sums, float) * 2.0 ** -60 / (3 * V * group), np.array(sizes, float) * 2.0 ** -60 / (3 * V * group)
+    poly = np.trace(L[3][0] @ L[3][1], axis1=-2, axis2=-1)
+    got, l = lat.measure()
+    assert (np.abs(np.array(got[1:]) - P) < 10 * 2.0 ** -53 * S).all(), (got, P)
+    assert abs(complex(*l) - poly.mean() / group) < 10 * 2.0 ** -53 * np.abs(poly).mean(), (l, poly.mean())
+    lat.close()
