@@ -735,7 +735,6 @@ struct SumD {
   double s = 0.0;
   __device__ __forceinline__ void add(double v) { s += v; }
   __device__ __forceinline__ void merge_down(int off) { s += __shfl_down_sync(0xffffffffu, s, off); }
-  __device__ __forceinline__ double value() const { return s; }
 };
 template <int N>
 __device__ __forceinline__ double warp_values(const SumD (&v)[N]) {

@@ -6,6 +6,8 @@
 // true there: links change inside that launch, so they are read through L2).
 #pragma once
 
+#include <type_traits>
+
 #include "qcd_kernels.cuh"
 
 namespace qcd {
@@ -162,7 +164,7 @@ __global__ void su2c_phase_kernel(const Ctx a, int parity) {
 template <typename R, bool FIELD, int MU>
 __global__ void su2c_or_meas_kernel(const Ctx a, int parity) {
   const int h = blockIdx.x * blockDim.x + threadIdx.x;
-  SumOf<R> v[1];
+  std::conditional_t<sizeof(R) == 4, SumF32, SumD> v[1];
   if (h < a.g.Vh) v[0].s = su2c_update<R, FIELD, KIND_OR_MEAS, MU, false>(a, parity, h, 0u);
   block_sums(v, a.partials + fused_plaq_offset(a.g, MU) + blockIdx.x);
 }

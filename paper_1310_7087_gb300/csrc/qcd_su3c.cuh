@@ -489,7 +489,7 @@ template <int FIELD, int MU>
 __global__ void __maxnreg__(QCD_SU3_MEAS_MAXNREG) su3c_or_meas_kernel(const Ctx a, int parity) {
   pdl_launch_dependents();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  SumF v[1];
+  SumF32 v[1];
   if (i < a.g.Vh) {
     const LexSite x = lex_site_ytz(a.g, parity, i);
     pdl_wait();
@@ -608,7 +608,7 @@ __global__ void __launch_bounds__(192, 3) su3c_split_kernel(const Ctx a, int par
     for (int sub = 0; sub < 3; ++sub)
       first[sub] = {sh.first[sub][0][lane], sh.first[sub][1][lane], sh.first[sub][2][lane],
                     sh.first[sub][3][lane], sh.first[sub][4][lane], sh.first[sub][5][lane]};
-  SumF v[1];
+  SumF32 v[1];
   if (on) {
     const M3<float> U = su3c_update<FIELD, KIND>(a, parity, mu, x.s >> 1, x, A, su3c_full(own), first, sweep);
     if (KIND == KIND_OR_MEAS) v[0].s = su3c_plane_sum<FIELD>(a, mu, x, U, low);

@@ -1,6 +1,6 @@
 """The sums of FP32 terms (qcd_sums.cuh) run by the host compiler: as close to the exact
 sum as FP64 can say (two roundings of it), for a thread's and a warp's worth of terms
-and for thousands of them; infinities and NaN as an FP64 sum gives them."""
+and for thousands of them (two numbers: for one term a lane); infinities and NaN as an FP64 sum gives them."""
 import os
 import subprocess
 
@@ -9,15 +9,17 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 PROGRAM = r"""
 #include "qcd_sums.cuh"
 #include <cstdio>
+#include <initializer_list>
 #include <random>
 using qcd::SumF;
-int main() {
+double worst = 0;
+template <class Sum>
+void sums(std::initializer_list<int> counts) {
   std::mt19937_64 g(1);
   std::uniform_real_distribution<float> u(0.f, 3.f);
-  double worst = 0;
-  for (int n : {1, 3, 6, 40, 1000, 20000})
+  for (int n : counts)
     for (int it = 0; it < (n > 100 ? 20 : 2000); ++it) {
-      SumF lane[32];
+      Sum lane[32];
       __int128 exact = 0, size = 0;  // units of 2^-40: the terms are multiples of it
       for (int l = 0; l < 32; ++l)
         for (int k = 0; k < n; ++k) {
@@ -34,6 +36,10 @@ int main() {
       const double err = double(d < 0 ? -d : d) / double(size << 20);
       if (err > worst) worst = err;
     }
+}
+int main() {
+  sums<SumF>({1, 3, 6, 40, 1000, 20000});
+  sums<qcd::SumF32>({1});
   SumF a, b, c, d;
   const float inf = HUGE_VALF;
   for (float v : {1.f, inf, 2.f}) a.add(v);
