@@ -167,10 +167,10 @@ QCD_HD int64_t fx_kp_a3(uint32_t w3) {
 }
 
 // Whether an accepted try's e (2^-57 units) is too small for fixed point: fx_kp_e is
-// right to about 2^-57, which the square root below magnifies; below 2^-15 (one
-// draw in 8 million: an FP64 update takes its warp 100 us) the update is left to FP64,
+// right to about 2^-57, which the square root below magnifies; below 2^-16 (one
+// draw in 22 million: an FP64 update takes its warp 100 us) the update is left to FP64,
 // whose error is relative.
-QCD_HD bool fx_kp_small(double e) { return uint32_t(fx_bits(e) >> 32) < uint32_t(1023 + FX_UNIT - 1 - 15) << 20; }
+QCD_HD bool fx_kp_small(double e) { return uint32_t(fx_bits(e) >> 32) < uint32_t(1023 + FX_UNIT - 1 - 16) << 20; }
 // delta = d 2^-57 of a try by the double's exponent and mantissa, m 2^(-63 - e) with m in
 // [2^63, 2^64): a small delta (weak coupling) keeps its bits.  e is negative for
 // delta >= 2, which no try accepts (infinities too).
@@ -248,8 +248,8 @@ __device__ __forceinline__ FxKpFirst fx_kp_first(const Stream& tries, const Stre
 // may have (any beta) are FP64's, so 1 / alpha and delta = e / alpha are formed there
 // (three FP64 instructions); the test and all that follows are fixed point again.
 // Error of the drawn quaternion against long double, largest / rms, in units of that
-// of the same expressions in double: 0.39 / 0.36 at alpha = 3, 0.72 / 0.20 at 10,
-// 0.60 / 0.18 at 100, 0.37 / 0.16 at 1e4 (with delta in 2^-58 units throughout and no
+// of the same expressions in double: 0.39 / 0.36 at alpha = 3, 0.97 / 0.20 at 10,
+// 0.76 / 0.18 at 100, 0.46 / 0.16 at 1e4 (with delta in 2^-58 units throughout and no
 // bound on e: 0.39 / 0.36, 0.9 / 0.20, 6.4 / 0.4, 190 / 5 over 2 million draws, and
 // 5, 52, 340, 16000 for e next to 0).
 enum { FX_DRAWN = 0, FX_EXHAUSTED = 1, FX_SMALL_DRAW = 2 };

@@ -217,4 +217,4 @@ int main() {
 }
 """)
     assert len(out) == 13 and all(float(v) <= 1.0 for v in out[:-1]), out
-    assert 0 <= int(out[-1]) < 5, out  # 2.1 million draws, one in 8 million expected
+    assert 0 <= int(out[-1]) < 5, out  # 2.1 million draws, one in 22 million expected
