@@ -80,9 +80,9 @@ extern "C" {
 /* Update kinds for qcd_phase. */
 #define QCD_HEATBATH 0
 #define QCD_OVERRELAX 1
-#define QCD_OVERRELAX_REUNIT 2  /* overrelaxation, then the FP64 reunitarization
-                                   of each updated link: the kernels of the
-                                   last pass of a sweep                      */
+#define QCD_OVERRELAX_REUNIT 2  /* overrelaxation, then the reunitarization of
+                                   each updated link: the kernels of the last
+                                   pass of a sweep                           */
 #define QCD_OVERRELAX_MEASURE 3 /* as QCD_OVERRELAX_REUNIT, and the plaquette
                                    sums of a working sweep's fused
                                    measurement (odd parity, mu >= 1 only)    */
@@ -160,8 +160,10 @@ int qcd_get_field_mode(qcd_lattice *lat, int *field_mode);
 int qcd_set_nhit(qcd_lattice *lat, int nhit);
 
 /* Sweep (sec. 3.3, sec. 5): n_heatbath times { one heat-bath pass; n_overrelax
- * overrelaxation passes; FP64 reunitarization of every link }.  A pass visits
- * the 8 checkerboard phases: parity even then odd, inside it mu = x,y,z,t.
+ * overrelaxation passes; reunitarization of every link }.  The reunitarization
+ * of FP32 links is FP64 (or as close to it); that of FP64 links next to
+ * unitary is fixed point to 2^-58, of others FP64.  A pass visits the 8
+ * checkerboard phases: parity even then odd, inside it mu = x,y,z,t.
  * The reunitarization is applied by the last overrelaxation pass's kernels
  * to each link right after its update in that pass (each link is updated
  * once per pass), so it costs no separate pass over the links; with
@@ -179,9 +181,9 @@ int qcd_sweep(qcd_lattice *lat, int n_heatbath, int n_overrelax, uint64_t seed);
  * overrelaxation pass: after the pass each plaquette of plane (mu, nu < mu)
  * contains exactly one odd mu-link, so the odd phases mu = 1, 2, 3 add
  * Re Tr(Ut A_nu) for nu < mu over their updated links (A_nu the staples of
- * plane (mu, nu); FP32: each warp adds its threads' values by error-free
- * TwoSum and finishes in FP64, the block adds its warps in FP64, and the final
- * sums take the 1/3) and no separate pass over the links is needed; otherwise
+ * plane (mu, nu); each warp adds its threads' values without rounding (FP32
+ * values by error-free TwoSum, fixed-point ones as integers), the block adds
+ * its warps in FP64, and the final sums take the 1/3) and no separate pass over the links is needed; otherwise
  * the measurement kernels run after the sweeps.  wait = 1: returns after the
  * results are on the host; wait = 0: host_out (page-locked for overlap) is
  * filled once the stream is synchronized. */
@@ -195,7 +197,7 @@ int qcd_working_sweep(qcd_lattice *lat, int n_heatbath, int n_overrelax,
  *                                 phases (no reunitarization);
  *   QCD_OVERRELAX_REUNIT          a phase of the last overrelaxation pass of a
  *                                 sweep: each updated link is reunitarized
- *                                 (sec. 5) in FP64 before it is stored;
+ *                                 (sec. 5) before it is stored;
  *   QCD_OVERRELAX_MEASURE         a plane-summing phase of a working sweep's
  *                                 last pass (parity 1, mu = 1, 2, 3; else
  *                                 QCD_ERR_INVALID_ARG): as QCD_OVERRELAX_REUNIT,
@@ -226,11 +228,15 @@ int qcd_measure_fused_finish(qcd_lattice *lat, double *host_out);
 /* FP64 reunitarization of every link. */
 int qcd_reunitarize(qcd_lattice *lat);
 
-/* Measurements on the effective links (sec. 1, sec. 5), FP64 sums:
+/* Measurements on the effective links (sec. 1, sec. 5), sums as close as FP64
+ * ones (FP32 terms are added in the warps by error-free TwoSum, which keeps the
+ * rounding errors in two further numbers, and in FP64 from there on):
  *   plaquette[3] = {P, P_s, P_t}: (1/N) Re Tr of the plaquette averaged over
  *     all 6V plaquettes, the 3V spatial ones (mu,nu < t) and the 3V temporal;
  *   polyakov[2] = {Re L, Im L}: (1/N) Tr of the ordered product of t-links
  *     t = 0..Nt-1, averaged over the Ns^3 spatial sites.
+ * Links are taken as they are stored, unitary or not (FP32 SU(3): rows 0 and 1,
+ * and row 2 = conj(row 0 x row 1)).
  * Either pointer may be NULL.  Host pointers; synchronizes the stream. */
 int qcd_measure(qcd_lattice *lat, double *plaquette, double *polyakov);
 /* The same plaquettes on the bare links U (they depend on the field). */
@@ -378,7 +384,7 @@ int qcd_batch_create(qcd_batch **out, int n, int group, const int *Ns,
 int qcd_batch_destroy(qcd_batch *b);
 
 /* n_sweeps sweeps of every lattice (each: 1 heat-bath pass, n_overrelax
- * overrelaxation passes, FP64 reunitarization, measurement) in one launch
+ * overrelaxation passes, reunitarization, measurement) in one launch
  * per wave (see qcd_batch_set_wave_bytes; one launch when the links fit L2).
  * meas_out: host double[n][n_sweeps][5] = {P, P_s, P_t, Re L, Im L} after each
  * sweep, or NULL.  The first call chooses the launch shape (autotune over 128,

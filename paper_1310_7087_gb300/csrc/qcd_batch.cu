@@ -265,8 +265,8 @@ __device__ void batch_run(const BatchArgs& b, int li, const BatchLat& L, int j) 
 #define QCD_BATCH_MAXNREG 64
 #endif
 
-// FP64 links take the fixed-point update (12.6 -> 4.8 ms per sweep of the
-// 64-lattice scan): 128 registers (4.9 ms; 112 / 96 / 80 / 64: 5.1 / 5.6 / 6.4 / 7.0),
+// FP64 links take the fixed-point update (12.6 -> 4.3 ms per sweep of the
+// 64-lattice scan): 128 registers (112 / 96 / 80 / 64: 1.04 / 1.14 / 1.31 / 1.43 times that),
 // and 64 where a wave has more lattices than CTAs of 128 are resident (each lattice
 // needs one: at 64 threads 1,216, with 64 registers 2,432).
 constexpr int BATCH_MAXNREG_F64 = 128;

@@ -10,13 +10,18 @@
 //
 // Error: 2^-58 absolute per quantised input and per product sum, against the
 // 2^-54 of each FP64 rounding of a number in [1/2, 1); sums of products are
-// exact between the two.
+// exact between the two.  (fx_load_int rounds towards zero and value() down, so the
+// errors have a sign, a sixteenth of the rounding that storing a result adds.)
 //
 // Ranges, above: for |v| < 2 a limb product is below 2^60 (hi hi') or 2^59 (hi lo'),
 // so a three-term complex dot product (6 real products per part, 12 cross
 // terms) stays below 2^62.6 in both accumulators.  fx_load reports the largest
-// exponent it saw and fx_check any result outside (-2, 2); a caller that finds
-// one (links that are not near unitary, infinities, NaN) takes its FP64 path.
+// exponent it saw and fx_check any result outside [-2, 2); a caller that finds
+// one (infinities and NaN among them) takes its FP64 path.  Below: a few 2^-58 are
+// less than FP64's rounding of numbers of order 1 only, so a staple sum, a subgroup
+// block, a link or a product whose parts are all small (fx_small, fx_small_block,
+// fx_tiny: links that are scaled down, next to never a sum that cancels) is left to
+// FP64 too.
 //
 // Plain C++ besides a few device instructions, so that the host
 // compiler can run the same arithmetic.

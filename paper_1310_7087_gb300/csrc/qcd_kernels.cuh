@@ -781,7 +781,7 @@ __device__ __forceinline__ void block_sums(Sum (&v)[N], double* out) {
 
 // ---------------------------------------------------------------------------
 // Measurements: plaquette (spatial / temporal split) and Polyakov loop.
-// Products in the storage precision, sums as above: per-thread value, warp
+// Products in the storage precision, sums by SumOf: per-thread value, warp
 // shuffle, per-block partial, then one block sums the partials in a fixed
 // order (deterministic for a given lattice).
 // ---------------------------------------------------------------------------

@@ -198,10 +198,9 @@ __device__ __forceinline__ double su2d_update_at(const Ctx& a, int parity, const
 // Bound: integer pipe and FP64 unit together (ncu at 32^3x8, overrelaxation of
 // t-links: ALU 45 %, 3,390 instructions per update) where the FP64 form was bound
 // by the FP64 unit.  Phase times, us, FP64 form -> this, overrelaxation /
-// heat-bath of y-links: 32^3x8 77 / 159 -> 31 / 45;
-// 64^3x16 1104 / 2135 -> 440 / 661.  128 registers: 96 / 80 / 64 gave sweeps of
-// 8.2 / 8.5 / 9.4 ms at 64^3x16 against 8.2, and 572 / 640 / 613 us at 32^3x8
-// against 534.
+// heat-bath of y-links: 32^3x8 77 / 159 -> 32 / 42;
+// 64^3x16 1104 / 2135 -> 406 / 529.  128 registers: with 96 / 80 / 64 sweeps took
+// 1.00 / 1.04 / 1.15 times as long at 64^3x16 and 1.07 / 1.20 / 1.15 at 32^3x8.
 //
 // One thread per link.
 template <bool FIELD, int KIND, int MU>
@@ -217,8 +216,8 @@ __global__ void __maxnreg__(128) su2d_phase_kernel(const __grid_constant__ Ctx a
 // sums are exact, so the results are the same.  The directions are run-time values
 // and the two kinds of staple one body (the adjoint of a link by the sign of its
 // imaginary quaternion parts), so that the code stays in the instruction caches
-// from phase to phase (a kernel per direction with a body per staple took 91 / 137 /
-// 160 us per sweep at 4^3x4 / 12^3x4 / 16^3x4, this one 84 / 95 / 104).
+// from phase to phase (a kernel per direction with a body per staple took 1.1 / 1.4 /
+// 1.5 times as long per sweep at 4^3x4 / 12^3x4 / 16^3x4).
 __device__ __forceinline__ void su2d_load_at(const Ctx& a, int d, int par, int s, uint32_t dag, Fx q[4], uint32_t& big) {
   const Quat<double> u = SU2Policy<double>::load(a.links, a.g, d, par, s >> 1);
   const double v[4] = {u.q0, u.q1, u.q2, u.q3};
@@ -311,8 +310,8 @@ __global__ void __launch_bounds__(192) su2d_split_kernel(const __grid_constant__
 }
 
 // Split up to 512 CTAs of 32 links: sweeps of 1 heat-bath + 1 overrelaxation pass,
-// us, split / not: 4^3x4 84 / 148, 12^3x4 (108 CTAs) 95 / 155, 16^3x4 (256) 104 / 158,
-// 20^3x4 (500) 156 / 162.
+// us, split / not: 4^3x4 71 / 130, 12^3x4 (108 CTAs) 82 / 142, 16^3x4 (256) 89 / 142,
+// 20^3x4 (500) 141 / 149.
 inline bool su2d_split(const GeomH& g) { return (g.Vh + 31) / 32 <= 512; }
 // Links of one CTA for a block size of the caller.
 inline int su2d_links_per_cta(const GeomH& g, int block) { return su2d_split(g) ? 32 : block; }

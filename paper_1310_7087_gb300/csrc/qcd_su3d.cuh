@@ -14,11 +14,12 @@
 // the multiplier's pipe 61 % busy, adds, shifts and logic the ALU 51 %; 21,200
 // warp instructions per 32 updates; fixed-latency waits and the pipes' are the
 // largest stalls) where the FP64 form was bound by the FP64 unit (94 % busy).
-// Overrelaxation / heat-bath phase, us, FP64 form -> this: 4^3x4 73.8 / 118.9 ->
-// 12 / 18; 16^3x4 75.8 / 126.2 -> 18 / 25; 32^3x8 447 / 710 -> 149 / 215; 48^3x16
-// 2868 / 4314 -> 915 / 1408.  One thread per link (168 registers) took 1231 us for
-// the last, with the matrices unrolled for both kinds of staple 1665 (instruction
-// cache); one copy of the subgroup rotation for all three 1 to 2 % more.
+// Overrelaxation / heat-bath phase of y-links, us, FP64 form -> this: 4^3x4 73.8 / 118.9
+// -> 12 / 16.5; 16^3x4 75.8 / 126.2 -> 18.5 / 25; 32^3x8 447 / 710 -> 151 / 214;
+// 48^3x16 2868 / 4314 -> 939 / 1408.  One thread per link (168 registers) took 1231 us
+// for the overrelaxation of the last, with the matrices unrolled for both kinds of
+// staple 1665 (instruction cache); applying the rotations to the rows by one copy of
+// the code for all three subgroups (finding them is one copy) 1 to 2 % more.
 #pragma once
 
 #include <type_traits>

@@ -105,8 +105,8 @@ __device__ __forceinline__ void su3d_plaquettes(const Ctx& a, int p, int base, S
 
 // Measurement of a configuration: CTAs of eight groups of three warps, 256 sites (as
 // measure_kernel's blocks, for the same partials): plaquettes, then the Polyakov loop.
-// Measurement at 16^3x4 / 32^3x8 / 48^3x16, us: 60 / 340 / 2190, against 128 / 772 /
-// 4880 by the FP64 kernel (SU(2), one thread a site: 24 / 66 / 396 against 42 / 159 / 898).
+// Measurement at 16^3x4 / 32^3x8 / 48^3x16, us: 60 / 344 / 2200, against 128 / 772 /
+// 4880 by the FP64 kernel (SU(2), one thread a site: 23 / 66 / 394 against 42 / 159 / 898).
 template <int FIELD>
 __global__ void __launch_bounds__(768) su3d_measure_kernel(const __grid_constant__ Ctx a, int n_plaq_blocks) {
   extern __shared__ __align__(16) unsigned char smem[];
