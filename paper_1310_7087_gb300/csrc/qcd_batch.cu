@@ -357,16 +357,16 @@ int* d_error(qcd_batch* B) { return reinterpret_cast<int*>(B->d_small + 4); }
 int* d_error_where(qcd_batch* B) { return reinterpret_cast<int*>(B->d_small + 8); }
 unsigned long long* d_exhausted(qcd_batch* B) { return reinterpret_cast<unsigned long long*>(B->d_small + 16); }
 
-void (*batch_kernel_ptr(const qcd_batch* B))(BatchArgs) {
+void (*batch_kernel_ptr(const qcd_batch* B, bool narrow))(BatchArgs) {
   if (B->precision != QCD_FP64_PLAIN) return qcd::batch_kernel<float, QCD_BATCH_MAXNREG>;
-  return B->narrow ? qcd::batch_kernel<double, QCD_BATCH_MAXNREG> : qcd::batch_kernel<double, qcd::BATCH_MAXNREG_F64>;
+  return narrow ? qcd::batch_kernel<double, QCD_BATCH_MAXNREG> : qcd::batch_kernel<double, qcd::BATCH_MAXNREG_F64>;
 }
 
 // Resident CTAs for a block size (cooperative launch needs all CTAs
 // resident), at most `per_sm_cap` per SM when that is > 0.
-int resident_ctas(qcd_batch* B, int block, int per_sm_cap) {
+int resident_ctas(const qcd_batch* B, int block, int per_sm_cap, bool narrow) {
   int per_sm = 0, sms = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel_ptr(B), block, 0) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel_ptr(B, narrow), block, 0) !=
           cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, B->device) != cudaSuccess) {
     cudaGetLastError();
@@ -455,7 +455,6 @@ std::vector<int> wave_starts(const qcd_batch* B) {
   l0.push_back(B->n);
   return l0;
 }
-void form_waves(qcd_batch* B) { B->wave_l0 = wave_starts(B); }
 
 void drop_batch_graphs(qcd_batch* B) {
   for (auto& g : B->graphs) cudaGraphExecDestroy(g.exec);
@@ -463,30 +462,35 @@ void drop_batch_graphs(qcd_batch* B) {
 }
 
 // Lay out the CTA groups of every wave for `block` threads (at most `per_sm`
-// CTAs per SM, 0 = as many as fit) and upload descriptors.
+// CTAs per SM, 0 = as many as fit) and upload descriptors.  A shape that does not
+// fit is refused before anything changes; from there on until all is in place the
+// batch has no launch shape (block 0).
 int configure(qcd_batch* B, int block, int per_sm = 0) {
-  form_waves(B);
+  const std::vector<int> l0 = wave_starts(B);
   int lattices = 0;  // of the fullest wave
-  for (size_t w = 0; w + 1 < B->wave_l0.size(); ++w) lattices = std::max(lattices, B->wave_l0[w + 1] - B->wave_l0[w]);
-  B->narrow = false;
-  int capacity = resident_ctas(B, block, per_sm);
+  for (size_t w = 0; w + 1 < l0.size(); ++w) lattices = std::max(lattices, l0[w + 1] - l0[w]);
+  bool narrow = false;
+  int capacity = resident_ctas(B, block, per_sm, narrow);
   if (capacity < lattices && B->precision == QCD_FP64_PLAIN) {
-    B->narrow = true;
-    capacity = resident_ctas(B, block, per_sm);
+    narrow = true;
+    capacity = resident_ctas(B, block, per_sm, narrow);
   }
+  if (capacity < lattices)
+    return batch_fail(QCD_ERR_NOT_SUPPORTED, "wave of " + std::to_string(lattices) + " lattices does not fit " +
+                                                 std::to_string(capacity) + " resident CTAs of " +
+                                                 std::to_string(block) + " threads");
+  drop_batch_graphs(B);
+  B->block = 0;
+  B->narrow = narrow;
+  B->wave_l0 = l0;
   std::vector<int> map;
   B->wave_cta0.clear();
   B->wave_ctas.clear();
   int largest = 0;
-  for (size_t w = 0; w + 1 < B->wave_l0.size(); ++w) {
+  for (size_t w = 0; w + 1 < l0.size(); ++w) {
     B->wave_cta0.push_back(int(map.size()));
-    const int got = allocate_ctas(B, block, capacity, B->wave_l0[w], B->wave_l0[w + 1], map);
-    if (got == 0)
-      return batch_fail(QCD_ERR_NOT_SUPPORTED, "wave of " + std::to_string(B->wave_l0[w + 1] - B->wave_l0[w]) +
-                                                   " lattices does not fit " + std::to_string(capacity) +
-                                                   " resident CTAs of " + std::to_string(block) + " threads");
-    B->wave_ctas.push_back(got);
-    largest = std::max(largest, got);
+    B->wave_ctas.push_back(allocate_ctas(B, block, capacity, l0[w], l0[w + 1], map));
+    largest = std::max(largest, B->wave_ctas.back());
   }
   if (size_t(largest) > B->partial_ctas) {
     if (B->d_partials) cudaFree(B->d_partials);
@@ -505,7 +509,6 @@ int configure(qcd_batch* B, int block, int per_sm = 0) {
   B->total_ctas = largest;
   B->block = block;
   B->per_sm = per_sm;
-  drop_batch_graphs(B);
   return QCD_OK;
 }
 
@@ -545,7 +548,7 @@ int enqueue(qcd_batch* B, const BatchArgs& a0, cudaStream_t st, bool advance) {
     BatchArgs a = a0;
     a.cta_lattice = B->d_cta + B->wave_cta0[w];
     void* params[] = {&a};
-    BATCH_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(batch_kernel_ptr(B)),
+    BATCH_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(batch_kernel_ptr(B, B->narrow)),
                                            dim3(B->wave_ctas[w]), dim3(B->block), params, 0, st));
   }
   if (advance) {
@@ -748,9 +751,12 @@ int qcd_batch_set_block(qcd_batch* B, int threads) {
 
 int qcd_batch_set_wave_bytes(qcd_batch* B, size_t bytes) {
   if (!B) return batch_fail(QCD_ERR_INVALID_ARG, "null batch");
+  const size_t before = B->wave_budget;
   B->wave_budget = bytes;
   if (B->block == 0) return QCD_OK;  // laid out with the launch shape on the next sweep
-  return configure(B, B->block, B->per_sm);
+  const int rc = configure(B, B->block, B->per_sm);
+  if (rc) B->wave_budget = before;
+  return rc;
 }
 
 int qcd_batch_get_waves(qcd_batch* B, int* waves, size_t* bytes) {
