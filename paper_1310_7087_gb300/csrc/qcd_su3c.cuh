@@ -625,9 +625,10 @@ __global__ void __launch_bounds__(192, 3) su3c_split_kernel(const Ctx a, int par
 // passes, us, not split / split: 4^3x4 229 / 113, 12^3x4 (108 CTAs) 230 / 127, 16^3x4
 // (256) 240 / 138, 20^3x4 (500) 231 / 222, 20^3x6 (750) 283 / 258, 22^3x6 (999) 311 / 332,
 // 24^3x6 (1296) 322 / 368.  (Up to two waves of 3 CTAs per SM, 912, it would still pay:
-// 24^3x4 (864) 336 / 266, 18^3x10 (912) 329 / 270.)  At these sizes a phase is one chain of latencies (one warp per SM
-// sub-partition or less): the gather's loads, 12 products one after another, the
-// update; the split takes the products and most of the loads out of the chain.
+// 24^3x4 (864) 336 / 266, 18^3x10 (912) 329 / 270.)  At these sizes a phase is one
+// chain of latencies (one warp per SM sub-partition or less): the gather's loads, 12
+// products one after another, the update; the split takes the products and most of
+// the loads out of the chain.
 inline bool su3c_split(const GeomH& g) { return (g.Vh + 31) / 32 <= 800; }
 // Links of one CTA for a block size of the caller.
 inline int su3c_links_per_cta(const GeomH& g, int block) { return su3c_split(g) ? 32 : block; }
